@@ -66,123 +66,103 @@ void plan_cg(Arena& a, CgWork& w, int32_t n, int32_t ld) {
 }
 
 
-// L_eps p_u = eps p_u + acc: store it (step/apply) or y_u minus it (residual), and add this
-// lane's column contributions to the dot partials (p.Ap, or |y - L x|^2)
-template <int LPR, int VPL, int MODE>
-__device__ __forceinline__ void finish_row(const SpmmArgs& a, int64_t u, int gl, int nvec,
-                                           const float4 (&pu)[VPL], const float4 (&acc)[VPL],
-                                           float2 (&dot)[VPL][4]) {
-#pragma unroll
-  for (int v = 0; v < VPL; ++v) {
-    const int q = gl + LPR * v;
-    if (q >= nvec) continue;
-    float4 o;
-    o.x = fmaf(a.eps, pu[v].x, acc[v].x);
-    o.y = fmaf(a.eps, pu[v].y, acc[v].y);
-    o.z = fmaf(a.eps, pu[v].z, acc[v].z);
-    o.w = fmaf(a.eps, pu[v].w, acc[v].w);
-    if (MODE == MODE_RESID) {
-      const float4 y = ld_f4(a.Y + (size_t)u * a.ld + 4 * q);
-      const int cb = 4 * q;
-      o.x = cb + 0 < a.kc ? y.x - o.x : 0.f;
-      o.y = cb + 1 < a.kc ? y.y - o.y : 0.f;
-      o.z = cb + 2 < a.kc ? y.z - o.z : 0.f;
-      o.w = cb + 3 < a.kc ? y.w - o.w : 0.f;
-      dot[v][0] = df_fma(dot[v][0], o.x, o.x);
-      dot[v][1] = df_fma(dot[v][1], o.y, o.y);
-      dot[v][2] = df_fma(dot[v][2], o.z, o.z);
-      dot[v][3] = df_fma(dot[v][3], o.w, o.w);
-    } else {
-      reinterpret_cast<float4*>(a.AP + (size_t)u * a.ld)[q] = o;
-      dot[v][0] = df_fma(dot[v][0], pu[v].x, o.x);
-      dot[v][1] = df_fma(dot[v][1], pu[v].y, o.y);
-      dot[v][2] = df_fma(dot[v][2], pu[v].z, o.z);
-      dot[v][3] = df_fma(dot[v][3], pu[v].w, o.w);
-    }
-  }
-}
+// One thread group per light row; the blocks' groups split the heavy rows, HB of them between two
+// barriers, and their slices are added in group order.  Rows wider than 128 columns are taken 128
+// columns at a time, so that a walk's registers hold 16 rows in flight whatever the width.
+// Two blocks an SM: 16 warps with 16 row loads each keep 128 KB in flight, which is what the
+// gathers can use.  Against one row at a time in batches of 8 with 24 warps an SM (before):
+// 169k nodes x 256 columns 315 -> 239 us, 233k x 32 1275 -> 776 us, 2.45M x 128 7.69 -> 7.20 ms
+// (there HBM bounds it: the gathers that miss L2), 2.45M x 32 2.18 -> 1.95 ms.
+constexpr int HB = 4;
+constexpr int U_SPMM = 16;
 
-template <int LPR, int VPL>
-__device__ __forceinline__ void load_row(const SpmmArgs& a, int64_t u, int gl, int nvec,
-                                         float4 (&pu)[VPL], float4 (&acc)[VPL]) {
-#pragma unroll
-  for (int v = 0; v < VPL; ++v) {
-    const int q = gl + LPR * v;
-    pu[v] = q < nvec ? ld_f4(a.P + (size_t)u * a.ld + 4 * q) : f4_zero();
-    acc[v] = f4_zero();
-  }
-}
-
-template <int LPR, int VPL, bool WEIGHTED, int MODE>
-__global__ void __launch_bounds__(T, VPL <= 2 ? 3 : VPL == 4 ? 2 : 1) k_spmm(SpmmArgs a) {
+template <int LPR, bool WEIGHTED, int MODE>
+__global__ void __launch_bounds__(T, 2) k_spmm(const __grid_constant__ SpmmArgs a) {
   // nothing left to do: no active column, or a bounded wait of the solve has given up
   if (MODE == MODE_STEP && (*(volatile int*)a.flags == 0 || *(volatile int*)(a.flags + 3) != 0))
     return;
-  __shared__ __align__(16) float smem[SMEM_FLOATS];
   constexpr int GPB = T / LPR;  // groups per block
+  __shared__ float4 part[HB][T];  // heavy-row slices, then the dot products' scratch
+  __shared__ float2 sbuf[MAX_LD];
+  __shared__ Slots<U_SPMM, WEIGHTED> slots[GPB];
   const int gl = threadIdx.x & (LPR - 1);
   const int gi = threadIdx.x / LPR;
   const int nvec = a.ld >> 2;
   const unsigned gm = group_mask<LPR>();
-  float2 dot[VPL][4];
-#pragma unroll
-  for (int v = 0; v < VPL; ++v)
-#pragma unroll
-    for (int t = 0; t < 4; ++t) dot[v][t] = make_float2(0.f, 0.f);
-
-  // heavy rows: one block per row, its GPB groups take equal slices of the neighbour list and
-  // group 0 adds the slices in group order
   const int64_t nheavy = a.nheavy ? *a.nheavy : 0;
-  for (int64_t h = blockIdx.x; h < nheavy; h += gridDim.x) {
-    const int64_t u = a.heavy[h];
-    const int64_t j0 = a.row_ptr[u], j1 = a.row_ptr[u + 1];
-    const int64_t per = (j1 - j0 + GPB - 1) / GPB;
-    const int64_t s0 = min(j1, j0 + gi * per), s1 = min(j1, s0 + per);
-    float4 pu[VPL], acc[VPL];
-    load_row<LPR, VPL>(a, u, gl, nvec, pu, acc);
-    gather_range<LPR, VPL, WEIGHTED>(a, a.P, gl, gm, 0, nvec, pu, s0, s1, acc);
-#pragma unroll
-    for (int v = 0; v < VPL; ++v) {
-      const int q = gl + LPR * v;
-      if (q < nvec) reinterpret_cast<float4*>(smem + gi * a.ld)[q] = acc[v];
-    }
-    __syncthreads();
-    if (gi == 0) {
-#pragma unroll
-      for (int v = 0; v < VPL; ++v) {
-        const int q = gl + LPR * v;
-        if (q >= nvec) continue;
-        float4 s = f4_zero();
-        for (int g = 0; g < GPB; ++g) {
-          const float4 c = reinterpret_cast<const float4*>(smem + g * a.ld)[q];
-          s.x += c.x;
-          s.y += c.y;
-          s.z += c.z;
-          s.w += c.w;
-        }
-        acc[v] = s;
+  const int hmine = nheavy > blockIdx.x ? (int)((nheavy - blockIdx.x + gridDim.x - 1) / gridDim.x) : 0;
+  const uint32_t u0 = blockIdx.x * GPB + gi, ustep = gridDim.x * GPB;
+  const int mine = (uint32_t)a.n > u0 ? (int)(((uint32_t)a.n - u0 + ustep - 1) / ustep) : 0;
+  for (int q0 = 0; q0 < nvec; q0 += LPR) {
+    const int q = q0 + gl;
+    const bool valid = q < nvec;
+    const float* Pq = a.P + 4 * (valid ? q : nvec - 1);  // a spare lane repeats the last quad
+    f32x2 hi[2] = {0, 0}, lo[2] = {0, 0};  // dot partials of this lane's four columns
+    auto own = [&](uint32_t u) { return ld_quad<false>(Pq + (size_t)u * a.ld); };
+    // L_eps p_u: store it (step/apply) or take y_u minus it (residual); p.Ap or |y - L x|^2
+    auto finish = [&](uint32_t u, Quad pu, Quad acc) {
+      if (!valid) return;
+      Quad o = apply_quad(a.eps, pu, acc);
+      const size_t at = (size_t)u * a.ld + 4 * q;
+      if (MODE == MODE_RESID) {
+        const float4 y = ld_f4(a.Y + at), s = unquad(o);
+        const int cb = 4 * q;
+        o = quad(make_float4(cb + 0 < a.kc ? y.x - s.x : 0.f, cb + 1 < a.kc ? y.y - s.y : 0.f,
+                             cb + 2 < a.kc ? y.z - s.z : 0.f, cb + 3 < a.kc ? y.w - s.w : 0.f));
+        pu = o;
+      } else {
+        *reinterpret_cast<float4*>(a.AP + at) = unquad(o);
       }
-      finish_row<LPR, VPL, MODE>(a, u, gl, nvec, pu, acc, dot);
+      df_fma2(hi[0], lo[0], pu.a, o.a);
+      df_fma2(hi[1], lo[1], pu.b, o.b);
+    };
+    for (int hb = 0; hb < hmine; hb += HB) {
+      const int cnt = min(HB, hmine - hb);
+      const int32_t* list = a.heavy + blockIdx.x + (size_t)hb * gridDim.x;
+      walk_rows<LPR, U_SPMM, WEIGHTED, false>(
+          a, Pq, gl, gm, slots[gi], cnt, true,
+          [&](int k, uint32_t& j, int& len, uint32_t& u) {
+            u = (uint32_t)__ldg(list + (size_t)k * gridDim.x);
+            heavy_slice(a.row_ptr, u, gi, GPB, j, len);
+          },
+          own, [&](int k, uint32_t, Quad, Quad acc) { part[k][threadIdx.x] = unquad(acc); });
+      __syncthreads();
+      for (int k = gi; k < cnt; k += GPB) {
+        const uint32_t u = (uint32_t)__ldg(list + (size_t)k * gridDim.x);
+        Quad sum = {0, 0};
+#pragma unroll 8
+        for (int g = 0; g < GPB; ++g) {
+          const Quad x = quad(part[k][g * LPR + gl]);
+          sum.a = add2(sum.a, x.a);
+          sum.b = add2(sum.b, x.b);
+        }
+        finish(u, own(u), sum);
+      }
+      __syncthreads();
+    }
+    walk_rows<LPR, U_SPMM, WEIGHTED, false>(
+        a, Pq, gl, gm, slots[gi], mine, true,
+        [&](int k, uint32_t& j, int& len, uint32_t& u) {
+          u = u0 + k * ustep;
+          uint32_t n;
+          row_slots(a.row_ptr, u, j, n);
+          len = n > (uint32_t)a.H ? -1 : (int)n;
+        },
+        own, [&](int, uint32_t u, Quad pu, Quad acc) { finish(u, pu, acc); });
+    if (MODE == MODE_APPLY && a.pap_out == nullptr) continue;
+    float2 dot[1][4];
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+      const float2 h = unpack2(hi[t]), l = unpack2(lo[t]);
+      dot[0][2 * t] = make_float2(h.x, l.x);
+      dot[0][2 * t + 1] = make_float2(h.y, l.y);
     }
     __syncthreads();
-  }
-
-  // light rows: one group per row
-  const int64_t ngroups = (int64_t)gridDim.x * GPB;
-  for (int64_t u = (int64_t)blockIdx.x * GPB + gi; u < a.n; u += ngroups) {
-    const int64_t j0 = a.row_ptr[u], j1 = a.row_ptr[u + 1];
-    if (j1 - j0 > a.H) continue;
-    float4 pu[VPL], acc[VPL];
-    load_row<LPR, VPL>(a, u, gl, nvec, pu, acc);
-    gather_range<LPR, VPL, WEIGHTED>(a, a.P, gl, gm, 0, nvec, pu, j0, j1, acc);
-    finish_row<LPR, VPL, MODE>(a, u, gl, nvec, pu, acc, dot);
+    block_partials_groups<LPR, 1, WARPS, 4 * LPR>(dot, sbuf + 4 * q0,
+                                                  reinterpret_cast<float2*>(&part[0][0]),
+                                                  min(4 * LPR, a.ld - 4 * q0));
   }
   if (MODE == MODE_APPLY && a.pap_out == nullptr) return;
-
-  float2* sbuf = reinterpret_cast<float2*>(smem);
-  float2* scratch = reinterpret_cast<float2*>(smem + 2 * MAX_LD);
-  __syncthreads();
-  block_partials_rowgroup<LPR, VPL>(dot, sbuf, scratch, a.ld);
   if (!grid_colreduce(a.cr, sbuf, sbuf, a.ld)) return;
   for (int c = threadIdx.x; c < a.ld; c += blockDim.x) {
     const double v = df_value(sbuf[c]);
@@ -1032,30 +1012,33 @@ __global__ void __launch_bounds__(HLT) k_list_heavy(const int64_t* __restrict__ 
 // ---------------------------------------------------------------------------- launch helpers
 inline int vec_threads(int nvec) { return nvec * (T / nvec); }
 
-template <int MODE>
-const void* spmm_kernel(int nvec, bool weighted) {
-  const void* k = nullptr;
-  dispatch_shape(nvec, [&](auto lpr, auto vpl) -> erc_status {
-    constexpr int LPR = decltype(lpr)::value, VPL = decltype(vpl)::value;
-    k = weighted ? (const void*)k_spmm<LPR, VPL, true, MODE>
-                 : (const void*)k_spmm<LPR, VPL, false, MODE>;
-    return ERC_OK;
-  });
-  return k;
+// calls f(ic<LPR>) for a row of nvec float4s
+template <class F>
+auto with_lpr(int nvec, F&& f) {
+  return nvec <= 4 ? f(ic<4>{}) : nvec <= 8 ? f(ic<8>{}) : nvec <= 16 ? f(ic<16>{}) : f(ic<32>{});
 }
 
-// grid and heavy threshold of the operator for this graph: one wave of blocks, and rows heavier
-// than about twice the mean work of a group are split over a block
+template <int MODE>
+const void* spmm_kernel(int nvec, bool weighted) {
+  return with_lpr(nvec, [&](auto lpr) -> const void* {
+    constexpr int LPR = decltype(lpr)::value;
+    return weighted ? (const void*)k_spmm<LPR, true, MODE> : (const void*)k_spmm<LPR, false, MODE>;
+  });
+}
+
+// grid and heavy threshold of the operator for this graph: one wave of blocks, and rows with more
+// neighbours than an eighth of a group's mean share go to whole blocks: on power-law graphs a
+// group that drew a row near the mean share would otherwise hold up its block long after the
+// others finished.  The share is taken over three blocks an SM, whatever the grid: the threshold
+// decides how a long row's sum is split, so it depends on the graph and the width alone.
+// Half and twice the threshold measured 255 and 247 us against 234 us (169k nodes x 256 columns),
+// 853 and 823 against 798 us (233k x 32).
 void spmm_shape(const erc_graph* g, int ld, int* grid, int32_t* H) {
   const int nvec = ld / 4;
-  int lpr = nvec <= 4 ? 4 : nvec <= 8 ? 8 : nvec <= 16 ? 16 : 32;
-  const int gpb = T / lpr;
-  *grid = one_wave_grid(spmm_kernel<MODE_STEP>(nvec, g->val != nullptr), T,
-                        ((long long)g->n + gpb - 1) / gpb);
-  // rows with more neighbours than an eighth of a group's mean share go to whole blocks: on
-  // power-law graphs a group that drew a row near the mean share would otherwise hold up its
-  // block long after the others finished
-  const long long groups = (long long)(*grid) * gpb;
+  const int gpb = T / with_lpr(nvec, [](auto lpr) { return (int)decltype(lpr)::value; });
+  const long long blocks = ((long long)g->n + gpb - 1) / gpb;
+  *grid = one_wave_grid(spmm_kernel<MODE_STEP>(nvec, g->val != nullptr), T, blocks);
+  const long long groups = std::min<long long>(blocks, 3LL * sm_count()) * gpb;
   long long h = 2 * g->m / (8 * groups);
   if (h < 32) h = 32;
   if (h > (1 << 20)) h = 1 << 20;
@@ -1076,12 +1059,12 @@ erc_status build_heavy(const erc_graph* g, int32_t H, const HeavyRows& hv, cudaS
 
 template <int MODE>
 erc_status launch_spmm(const SpmmArgs& a, int grid, cudaStream_t s) {
-  return dispatch_shape(a.ld / 4, [&](auto lpr, auto vpl) -> erc_status {
-    constexpr int LPR = decltype(lpr)::value, VPL = decltype(vpl)::value;
+  return with_lpr(a.ld / 4, [&](auto lpr) -> erc_status {
+    constexpr int LPR = decltype(lpr)::value;
     if (a.val)
-      k_spmm<LPR, VPL, true, MODE><<<grid, T, 0, s>>>(a);
+      k_spmm<LPR, true, MODE><<<grid, T, 0, s>>>(a);
     else
-      k_spmm<LPR, VPL, false, MODE><<<grid, T, 0, s>>>(a);
+      k_spmm<LPR, false, MODE><<<grid, T, 0, s>>>(a);
     count_launches(1);
     ERC_CUDA(cudaGetLastError());
     return ERC_OK;
@@ -1111,7 +1094,6 @@ erc_status launch_update(const VecArgs& va, int grid, cudaStream_t s) {
 }
 
 // ---- resident path selection: the kernel for this shape, its shared memory, and whether it fits
-int resident_lpr(int nvec) { return nvec <= 4 ? 4 : nvec <= 8 ? 8 : nvec <= 16 ? 16 : 32; }
 
 // the resident kernel for this shape (null where the row block is too wide for it); the
 // preconditioned instantiations live in their own translation unit
@@ -1154,20 +1136,22 @@ size_t open_smem(const void* k) {
 // shared memory of the resident kernel: r, Ap (and p with PS) of `rows` rows, the column
 // partials, the region shared by the heavy-row slices and the reduction scratch, and the local
 // heavy-row list
-size_t resident_smem(int64_t rows, int ld, bool ps) {
-  const size_t shared = resident_shared_floats_for(PT / resident_lpr(ld / 4), ld);
-  return 4 * ((ps ? 3 : 2) * (size_t)rows * ld + 2 * (size_t)ld + shared + (size_t)rows);
+size_t resident_smem(int64_t rows, int ld, bool ps, int hrows) {
+  return 4 * ((ps ? 3 : 2) * (size_t)rows * ld + 2 * (size_t)ld + resident_shared_floats(hrows) +
+              (size_t)rows);
 }
 
-bool resident_plan(const erc_graph* g, int ld, bool pc, int32_t* rb, size_t* smem,
-                   const void** kern) {
+bool resident_plan(const erc_graph* g, int ld, bool pc, int32_t* rb, int32_t* hrows,
+                   size_t* smem, const void** kern) {
   const int nvec = ld / 4;
   const int grid = sm_count();
   const int64_t rows = ((int64_t)g->n + grid - 1) / grid;
   for (int ps = 1; ps >= 0; --ps) {  // p in shared memory when it fits
     const void* k = resident_kernel(nvec, g->val != nullptr, ps, pc);
     if (!k) return false;
-    const size_t bytes = resident_smem(rows, ld, ps);
+    int hr = 8;  // heavy rows between two barriers: as many as the memory left over holds
+    while (hr > 1 && resident_smem(rows, ld, ps, hr) > open_smem(k)) hr /= 2;
+    const size_t bytes = resident_smem(rows, ld, ps, hr);
     if (bytes > open_smem(k)) continue;
     int nb = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, PT, bytes) != cudaSuccess || nb < 1) {
@@ -1175,6 +1159,7 @@ bool resident_plan(const erc_graph* g, int ld, bool pc, int32_t* rb, size_t* sme
       continue;
     }
     *rb = (int32_t)rows;
+    *hrows = hr;
     *smem = bytes;
     *kern = k;
     return true;
@@ -1263,7 +1248,7 @@ bool cluster_plan(const erc_graph* g, int ld, ClusterPlan* pl) {
 struct SolverPlans {
   bool cluster = false, resident = false;
   ClusterPlan cp;
-  int32_t rb = 0;
+  int32_t rb = 0, hrows = 1;
   size_t smem = 0;
   const void* kres = nullptr;
 };
@@ -1289,7 +1274,7 @@ SolverPlans solver_plans(const erc_graph* g, int ld, bool pc) {
   }
   SolverPlans p;
   p.cluster = !pc && cluster_plan(g, ld, &p.cp);  // the cluster solver has no preconditioner
-  p.resident = resident_plan(g, ld, pc, &p.rb, &p.smem, &p.kres);
+  p.resident = resident_plan(g, ld, pc, &p.rb, &p.hrows, &p.smem, &p.kres);
   std::lock_guard<std::mutex> lock(mu);
   Entry& e = cache[next];
   next = (next + 1) % 16;
@@ -1566,7 +1551,7 @@ erc_status erc::cg_enqueue(const erc_graph* g, float eps, const float* Y, float*
     ERC_TRY(launch_cluster(cp, ca, s));
   } else if (resident) {
     // the whole solve in one cooperative launch, no host round trips
-    ResArgs ra{sa, va, rb};
+    ResArgs ra{sa, va, rb, plans.hrows};
     ra.v.spin_limit = wait_limit(RES_SPIN_LIMIT);
     ERC_TRY(launch_resident(kres, ra, smem, s));
   } else {

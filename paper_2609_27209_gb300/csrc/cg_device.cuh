@@ -11,7 +11,6 @@ namespace {
 
 constexpr int T = 256;
 constexpr int WARPS = T / 32;
-constexpr int SMEM_FLOATS = 8192;  // 32 KB: heavy-row combine buffer, or the reduction buffers
 // default poll limits of the bounded waits: the vector update's grid barrier (which sleeps 64 ns
 // between polls) and the resident solver's synchronisations (one L2 round trip per poll); either
 // is seconds, far beyond any legitimate wait
@@ -87,95 +86,208 @@ __device__ __forceinline__ void block_partials_groups(float2 (&d)[VPL][4], float
   }
 }
 
-// per-warp then per-block combination of per-thread column partials of a row-group kernel
-template <int LPR, int VPL>
-__device__ __forceinline__ void block_partials_rowgroup(float2 (&d)[VPL][4], float2* sbuf,
-                                                        float2* scratch, int ld) {
+// ---------------------------------------------------------------------------- the row walk
+// Two float32 values in a 64-bit register, and the packed operations on them: each half is rounded
+// as the scalar operation rounds it, at half the issue slots.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(f32x2 v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+// a - b: the product with -1 is exact, so the one rounding is the difference's
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) { return fma2(b, pack2(-1.f, -1.f), a); }
+
+// df_fma on two columns at once: (hi, lo) += a b
+__device__ __forceinline__ void df_fma2(f32x2& hi, f32x2& lo, f32x2 a, f32x2 b) {
+  const f32x2 p = mul2(a, b), pe = fma2(a, b, mul2(p, pack2(-1.f, -1.f)));
+  const f32x2 s = add2(hi, p), bb = sub2(s, hi);
+  f32x2 e = add2(sub2(hi, sub2(s, bb)), sub2(p, bb));
+  e = add2(e, add2(lo, pe));
+  hi = add2(s, e);
+  lo = sub2(e, sub2(hi, s));
+}
+
+// four consecutive columns of a row
+struct Quad {
+  f32x2 a, b;
+};
+__device__ __forceinline__ Quad quad(float4 v) { return Quad{pack2(v.x, v.y), pack2(v.z, v.w)}; }
+__device__ __forceinline__ float4 unquad(Quad q) {
+  const float2 x = unpack2(q.a), y = unpack2(q.b);
+  return make_float4(x.x, x.y, y.x, y.y);
+}
+template <bool L2ONLY>
+__device__ __forceinline__ Quad ld_quad(const float* p) {
+  return quad(L2ONLY ? __ldcg(reinterpret_cast<const float4*>(p)) : ld_f4(p));
+}
+
+// The neighbour ids (and weights) of two steps of a group, in shared memory: a step reads four at a
+// time, where lanes that passed each other the ids would take a shuffle for every slot.
+template <int U, bool WEIGHTED>
+struct alignas(16) Slots {
+  uint32_t id[2][U];
+  float w[WEIGHTED ? 2 : 1][WEIGHTED ? U : 4];
+};
+
+// A group of LPR lanes walks a list of `nrows` rows, four columns a lane: row k's sum over its
+// neighbours, acc = sum_j w_j (p_u - p_{col_j}) in CSR order, goes to emit(k, u, p_u, acc).
+// bounds(k, start, len, u) names row k: its id and the CSR slots [start, start + len) to sum, len
+// < 0 for a row that is not this walk's to emit.  own(u) is this lane's quad of p_u; srcq is
+// column-quad address of row 0.  L2ONLY loads p through L2 only: required where p is rewritten
+// within the same launch.  A lane with `on` false loads no neighbour (own must give it zero).
+//
+// The gathers are random row reads that L2 serves at up to 20 TB/s (64 bytes a clock and SM), if
+// enough of them are in flight: what bounds a walk is the latency of the chain row bounds ->
+// neighbour ids -> neighbour rows.  So the chain is taken apart: a step gathers up to U rows at
+// once, and while they are on their way the next step's ids are loaded, which at a row's end are
+// the next row's first, and the bounds of the row after that.  The short last step of a row takes 4,
+// 8 or U slots; those past the end hold the row itself, which is cached and adds exactly zero
+// (loads that are predicated off or replaced by p_u measured up to 13% slower over a solve).
+template <int LPR, int U, bool WEIGHTED, bool L2ONLY, class Bounds, class Own, class Emit>
+__device__ __forceinline__ void walk_rows(const SpmmArgs& a, const float* __restrict__ srcq,
+                                          int gl, unsigned gm, Slots<U, WEIGHTED>& slots,
+                                          int nrows, bool on, Bounds&& bounds, Own&& own,
+                                          Emit&& emit) {
+  constexpr int E = (U + LPR - 1) / LPR;  // ids a lane fetches
+  const uint32_t ld = (uint32_t)a.ld;
+  auto put = [&](int b, const uint32_t(&c)[E], const float(&w)[E]) {
 #pragma unroll
-  for (int off = LPR; off < 32; off <<= 1) {
+    for (int e = 0; e < E; ++e) {
+      const int k = gl + e * LPR;
+      if (U % LPR != 0 && k >= U) continue;
+      slots.id[b][k] = c[e];
+      if (WEIGHTED) slots.w[b][k] = w[e];
+    }
+  };
+  auto fetch = [&](uint32_t u, uint32_t j, int rem, uint32_t(&c)[E], float(&w)[E]) {
 #pragma unroll
-    for (int v = 0; v < VPL; ++v)
-#pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        float2 o;
-        o.x = __shfl_xor_sync(0xffffffffu, d[v][t].x, off);
-        o.y = __shfl_xor_sync(0xffffffffu, d[v][t].y, off);
-        d[v][t] = df_add(d[v][t], o);
+    for (int e = 0; e < E; ++e) {
+      const int k = gl + e * LPR;
+      c[e] = u;
+      w[e] = 0.f;
+      if (k < U && k < rem) {
+        c[e] = (uint32_t)__ldg(a.col + (size_t)(j + (uint32_t)k));
+        if (WEIGHTED) w[e] = __ldg(a.val + (size_t)(j + (uint32_t)k));
       }
-  }
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int cb = 0; cb < ld; cb += 256) {
-    if (lane < LPR) {
+    }
+  };
+  uint32_t u = 0, nu = 0, j = 0, nj = 0;  // slots are below 2^32: m < 2^31
+  int rem = -1, nrem = -1;
+  if (nrows > 0) bounds(0, j, rem, u);
+  if (nrows > 1) bounds(1, nj, nrem, nu);
+  uint32_t c[E];
+  float w[E];
+  int b = 0;  // the buffer that holds this step's slots
+  fetch(u, j, rem, c, w);
+  __syncwarp(gm);  // the group is done with the slots of an earlier walk
+  put(0, c, w);
+  __syncwarp(gm);
+  Quad pu = {0, 0}, acc = {0, 0};
+  bool fresh = true;
+  for (int k = 0; k < nrows;) {
+    const bool last = rem <= U;
+    fetch(last ? nu : u, last ? nj : j + U, last ? nrem : rem - U, c, w);
+    uint32_t bj = 0, bu = 0;
+    int brem = -1;
+    if (last && k + 2 < nrows) bounds(k + 2, bj, brem, bu);
+    if (fresh) pu = own(u);
+    auto step = [&](auto count) {
+      constexpr int N = decltype(count)::value;
+      Quad v[N];
 #pragma unroll
-      for (int v = 0; v < VPL; ++v)
+      for (int t = 0; t < N; t += 4) {
+        const uint4 id = *reinterpret_cast<const uint4*>(&slots.id[b][t]);
+        const uint32_t ids[4] = {id.x, id.y, id.z, id.w};
 #pragma unroll
-        for (int t = 0; t < 4; ++t) {
-          const int c = 4 * (lane + LPR * v) + t;
-          if (c >= cb && c < cb + 256 && c < ld) scratch[warp * 256 + (c - cb)] = d[v][t];
+        for (int r = 0; r < 4; ++r)
+          v[t + r] = on ? ld_quad<L2ONLY>(srcq + (size_t)ids[r] * ld) : Quad{0, 0};
+      }
+#pragma unroll
+      for (int t = 0; t < N; t += 4) {
+        float4 wq = make_float4(1.f, 1.f, 1.f, 1.f);
+        if constexpr (WEIGHTED) wq = *reinterpret_cast<const float4*>(&slots.w[b][t]);
+        const float ws[4] = {wq.x, wq.y, wq.z, wq.w};
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          const f32x2 da = sub2(pu.a, v[t + r].a), db = sub2(pu.b, v[t + r].b);
+          if (WEIGHTED) {
+            const f32x2 w2 = pack2(ws[r], ws[r]);
+            acc.a = fma2(w2, da, acc.a);
+            acc.b = fma2(w2, db, acc.b);
+          } else {
+            acc.a = add2(acc.a, da);
+            acc.b = add2(acc.b, db);
+          }
         }
+      }
+    };
+    if (rem > 0) {
+      if (rem <= 4) step(ic<4>{});
+      else if (U > 8 && rem <= 8) step(ic<8>{});
+      else step(ic<U>{});
     }
-    __syncthreads();
-    for (int c = threadIdx.x; c < 256 && cb + c < ld; c += blockDim.x) {
-      float2 acc = make_float2(0.f, 0.f);
-      for (int w = 0; w < WARPS; ++w) acc = df_add(acc, scratch[w * 256 + c]);
-      sbuf[cb + c] = acc;
+    put(b ^ 1, c, w);  // last read one step ago, before that step's barrier
+    if (last) {
+      if (rem >= 0) emit(k, u, pu, acc);
+      acc = Quad{0, 0};
+      ++k;
+      u = nu;
+      j = nj;
+      rem = nrem;
+      nu = bu;
+      nj = bj;
+      nrem = brem;
+    } else {
+      j += U;
+      rem -= U;
     }
-    __syncthreads();
+    fresh = last;
+    b ^= 1;
+    __syncwarp(gm);
   }
 }
 
-// acc += sum_{j in [j0, j1)} w_j (p_u - p_{col_j}) for this lane's float4 column slots
-// q = qb + gl + LPR v < qend whose bit v of `on` is set (the others keep acc); p is the n x ld
-// block src_rows.  L2ONLY loads p through L2 only: required where p is rewritten
-// within the same launch.
-template <int LPR, int VPL, bool WEIGHTED, bool L2ONLY = false, int UB = 8>
-__device__ __forceinline__ void gather_range(const SpmmArgs& a, const float* __restrict__ src_rows,
-                                             int gl, unsigned gm, int qb, int qend,
-                                             const float4 (&pu)[VPL], int64_t j0, int64_t j1,
-                                             float4 (&acc)[VPL], unsigned on = ~0u) {
-  constexpr int U = VPL >= UB ? 1 : UB / VPL;  // neighbour rows in flight per group
-  for (int64_t jb = j0; jb < j1; jb += LPR) {
-    const int64_t jj = jb + gl;
-    int32_t cidx = 0;
-    float wv = 1.f;
-    if (jj < j1) {
-      cidx = __ldg(a.col + jj);
-      if (WEIGHTED) wv = __ldg(a.val + jj);
-    }
-    const int cnt = (int)min((int64_t)LPR, j1 - jb);
-    // batches of U neighbour rows, the last one predicated: every load of a batch is issued
-    // before the first FMA, so a row costs ceil(deg / U) dependent trips
-    for (int t = 0; t < cnt; t += U) {
-      int cj[U];
-      float wj[U];
-      float4 pv[U][VPL];
-#pragma unroll
-      for (int k = 0; k < U; ++k) {
-        cj[k] = __shfl_sync(gm, cidx, (t + k) & (LPR - 1), LPR);
-        wj[k] = WEIGHTED ? __shfl_sync(gm, wv, (t + k) & (LPR - 1), LPR) : 1.f;
-        if (t + k >= cnt) wj[k] = 0.f;
-      }
-#pragma unroll
-      for (int k = 0; k < U; ++k)
-#pragma unroll
-        for (int v = 0; v < VPL; ++v) {
-          const int q = qb + gl + LPR * v;
-          const float* src = src_rows + (size_t)cj[k] * a.ld + 4 * q;
-          pv[k][v] = (q < qend && t + k < cnt && ((on >> v) & 1u))
-                         ? (L2ONLY ? __ldcg(reinterpret_cast<const float4*>(src)) : ld_f4(src))
-                         : pu[v];
-        }
-#pragma unroll
-      for (int k = 0; k < U; ++k)
-#pragma unroll
-        for (int v = 0; v < VPL; ++v) {
-          acc[v].x = fmaf(wj[k], pu[v].x - pv[k][v].x, acc[v].x);
-          acc[v].y = fmaf(wj[k], pu[v].y - pv[k][v].y, acc[v].y);
-          acc[v].z = fmaf(wj[k], pu[v].z - pv[k][v].z, acc[v].z);
-          acc[v].w = fmaf(wj[k], pu[v].w - pv[k][v].w, acc[v].w);
-        }
-    }
-  }
+// the CSR slots of row u
+__device__ __forceinline__ void row_slots(const int64_t* row_ptr, int64_t u, uint32_t& j,
+                                          uint32_t& len) {
+  j = (uint32_t)__ldg(row_ptr + u);
+  len = (uint32_t)__ldg(row_ptr + u + 1) - j;
+}
+// slice s of `parts` equal ones of a heavy row's slots
+__device__ __forceinline__ void heavy_slice(const int64_t* row_ptr, int64_t u, int s, int parts,
+                                            uint32_t& j, int& len) {
+  uint32_t j0, n;
+  row_slots(row_ptr, u, j0, n);
+  const uint32_t per = (n + parts - 1) / parts;
+  const uint32_t s0 = min(n, s * per), s1 = min(n, s0 + per);
+  j = j0 + s0;
+  len = (int)(s1 - s0);
+}
+// eps p_u + acc
+__device__ __forceinline__ Quad apply_quad(float eps, Quad pu, Quad acc) {
+  const f32x2 e = pack2(eps, eps);
+  return Quad{fma2(e, pu.a, acc.a), fma2(e, pu.b, acc.b)};
 }
 
 // the vectors and per-column state of one batched solve
@@ -214,6 +326,13 @@ __device__ __forceinline__ float4 f4_scale(float4 v, float s) {
 //   A  Ap = L_eps p on own rows (heavy rows by the whole block), p.Ap    -> reduce: alpha
 //   B  x += alpha p, r -= alpha Ap, r.r                                  -> reduce: beta, stop
 //   C  p = r + beta p                                                    -> barrier
+// Where node ids follow the degree (power-law graphs often come so), contiguous ranges give the
+// first block the hubs and every other block waits for it in A.  Such a solve runs A on dealt
+// rows instead (block b takes rows b, b + G, ...) and hands Ap to the owners through global
+// memory: the reduction of p.Ap between A and B orders the hand-over, so it costs no further
+// synchronisation.  B, C and their sums keep their blocks.  A 60,013-node power-law graph (411k
+// edges, 36 columns, Jacobi) took 14.2 ms a solve on its contiguous ranges and takes 1.7 ms; the
+// even 20,000-node graph of 128 columns keeps its ranges (1.49 ms then, 1.41 ms with the walk).
 // A grid synchronisation is an arrival (a release-add on a counter after the block's partials
 // are written) and a bounded wait until all blocks have arrived.  There is no finishing block:
 // after a reduction every block sums all blocks' partials itself, in the same fixed order, so
@@ -230,12 +349,16 @@ constexpr int PWARPS = PT / 32;
 constexpr int PCH = 64;
 constexpr int RMAXLD = 256;  // widest row block the resident kernel takes (64 float4)
 constexpr int RU = 2;  // float4 loads per lane in flight in phases B and C
-constexpr int RUB = 8;  // neighbour rows in flight per row group in the gathers
+// neighbour rows in flight per row group in the gathers (fewer for the narrowest rows, whose many
+// groups would otherwise take 32 KB of shared memory for their slots)
+template <int LPR>
+constexpr int RUB = LPR == 4 ? 8 : 16;
 
 struct ResArgs {
   SpmmArgs s;
   VecArgs v;
-  int32_t rb;  // rows per block
+  int32_t rb;     // rows per block
+  int32_t hrows;  // heavy rows whose slices the shared memory holds at once
 };
 
 __device__ __forceinline__ float4 ldcg_f4(const float* p) {
@@ -263,100 +386,73 @@ __device__ __forceinline__ void res_wait(const unsigned* arr, unsigned target, i
   __syncthreads();
 }
 
-// floats of the region shared by the heavy-row slices [GPB][ld] and the reduction scratch
-// [2 * PT float pairs] of the resident kernel
-__host__ __device__ constexpr size_t resident_shared_floats_for(int gpb, int ld) {
-  return (size_t)gpb * ld > 4 * (size_t)PT ? (size_t)gpb * ld : 4 * (size_t)PT;
-}
-__device__ __forceinline__ size_t resident_shared_floats(int ld) {
-  const int nvec = ld >> 2;
-  const int lpr = nvec <= 4 ? 4 : nvec <= 8 ? 8 : nvec <= 16 ? 16 : 32;
-  return resident_shared_floats_for(PT / lpr, ld);
+// floats of the region that the resident kernel uses for the heavy-row slices, `hrows` rows of one
+// quad per thread, and, after the operator, as the reduction scratch [2 * PT float pairs]
+__host__ __device__ constexpr size_t resident_shared_floats(int hrows) {
+  return 4 * (size_t)PT * (size_t)hrows;
 }
 
-// o = L_eps s on the block's rows, s = src_rows (n x ld; the block's own rows are read from `own`
-// when it is not null): o_u = eps s_u + sum_v w_uv (s_u - s_v).  The block's rows heavier than
-// a.H (the ascending local list hv[0..nh)) are split over all its groups and combined in group
-// order; the others take one group each.  emit(i, v, s_u, o_u) runs once per row i and valid
-// float4 slot v of the lane (for heavy rows in group 0).  Slots whose bit in `on` is clear are
-// neither loaded nor gathered (s_u = 0 there).
-template <int LPR, int VPL, bool WEIGHTED, class Emit>
-__device__ __forceinline__ void block_apply(const SpmmArgs& a, const float* src_rows,
-                                            const float* own, int64_t r0, int nrows,
-                                            const int* hv, int nh, float* comb, int gl, int gi,
-                                            unsigned gm, unsigned on, Emit&& emit) {
+// o = L_eps s on the rows r0 + i rstep, i < nrows, of s = src (n x ld): o_u = eps s_u +
+// sum_v w_uv (s_u - s_v).  own(u, v) is float4 slot v of the lane of s_u.  The rows heavier than
+// a.H (the ascending list hv[0..nh) of their i) are split over all groups of the block, hrows of
+// them between two barriers, and their slices are added in group order; the others take one group
+// each.  emit(i, u, v, s_u, o_u) runs once per row and valid slot.  Slots whose bit in `on` is
+// clear are neither loaded nor gathered (s_u = 0 there).
+template <int LPR, int VPL, bool WEIGHTED, class Own, class Emit>
+__device__ __forceinline__ void block_apply(const SpmmArgs& a, const float* src, int64_t r0,
+                                            int64_t rstep, int nrows, const int* hv, int nh,
+                                            int hrows, float* comb,
+                                            Slots<RUB<LPR>, WEIGHTED>& slots, int gl, int gi,
+                                            unsigned gm, unsigned on, Own&& own, Emit&& emit) {
   constexpr int GPB = PT / LPR;
-  const int ld = a.ld, nvec = ld >> 2;
-  auto own_row = [&](int i, int v) -> float4 {
+  const int nvec = a.ld >> 2;
+  float4* part = reinterpret_cast<float4*>(comb);  // [hrows][PT]
+#pragma unroll
+  for (int v = 0; v < VPL; ++v) {
     const int q = gl + LPR * v;
-    if (q >= nvec || !((on >> v) & 1u)) return f4_zero();
-    return own ? reinterpret_cast<const float4*>(own + (size_t)i * ld)[q]
-               : ldcg_f4(src_rows + (size_t)(r0 + i) * ld + 4 * q);
-  };
-  for (int hh = 0; hh < nh; ++hh) {
-    const int i = hv[hh];
-    const int64_t u = r0 + i;
-    const int64_t j0 = a.row_ptr[u], j1 = a.row_ptr[u + 1];
-    const int64_t per = (j1 - j0 + GPB - 1) / GPB;
-    const int64_t s0 = min(j1, j0 + gi * per), s1 = min(j1, s0 + per);
-    float4 pu[VPL], acc[VPL];
-#pragma unroll
-    for (int v = 0; v < VPL; ++v) {
-      pu[v] = own_row(i, v);
-      acc[v] = f4_zero();
-    }
-    gather_range<LPR, VPL, WEIGHTED, true, RUB>(a, src_rows, gl, gm, 0, nvec, pu, s0, s1, acc, on);
-#pragma unroll
-    for (int v = 0; v < VPL; ++v) {
-      const int q = gl + LPR * v;
-      if (q < nvec) reinterpret_cast<float4*>(comb + gi * ld)[q] = acc[v];
-    }
-    __syncthreads();
-    if (gi == 0) {
-#pragma unroll
-      for (int v = 0; v < VPL; ++v) {
-        const int q = gl + LPR * v;
-        if (q >= nvec) continue;
-        float4 s = f4_zero();
+    const bool valid = q < nvec, lane_on = valid && ((on >> v) & 1u);
+    const float* srcq = src + 4 * (valid ? q : 0);
+    auto own_quad = [&](uint32_t u) { return lane_on ? quad(own((int64_t)u, v)) : Quad{0, 0}; };
+    for (int hb = 0; hb < nh; hb += hrows) {
+      const int cnt = min(hrows, nh - hb);
+      walk_rows<LPR, RUB<LPR>, WEIGHTED, true>(
+          a, srcq, gl, gm, slots, cnt, lane_on,
+          [&](int k, uint32_t& j, int& len, uint32_t& u) {
+            u = (uint32_t)(r0 + hv[hb + k] * rstep);
+            heavy_slice(a.row_ptr, u, gi, GPB, j, len);
+          },
+          own_quad,
+          [&](int k, uint32_t, Quad, Quad acc) { part[k * PT + threadIdx.x] = unquad(acc); });
+      __syncthreads();
+      for (int k = gi; k < cnt; k += GPB) {
+        const int i = hv[hb + k];
+        const int64_t u = r0 + i * rstep;
+        const Quad pu = own_quad((uint32_t)u);
+        Quad sum = {0, 0};
+#pragma unroll 8
         for (int g = 0; g < GPB; ++g) {
-          const float4 c = reinterpret_cast<const float4*>(comb + g * ld)[q];
-          s.x += c.x;
-          s.y += c.y;
-          s.z += c.z;
-          s.w += c.w;
+          const Quad x = quad(part[k * PT + g * LPR + gl]);
+          sum.a = add2(sum.a, x.a);
+          sum.b = add2(sum.b, x.b);
         }
-        float4 o;
-        o.x = fmaf(a.eps, pu[v].x, s.x);
-        o.y = fmaf(a.eps, pu[v].y, s.y);
-        o.z = fmaf(a.eps, pu[v].z, s.z);
-        o.w = fmaf(a.eps, pu[v].w, s.w);
-        emit(i, v, pu[v], o);
+        if (valid) emit(i, u, v, unquad(pu), unquad(apply_quad(a.eps, pu, sum)));
       }
+      __syncthreads();
     }
-    __syncthreads();
-  }
-  for (int i = gi; i < nrows; i += GPB) {
-    const int64_t u = r0 + i;
-    const int64_t j0 = a.row_ptr[u], j1 = a.row_ptr[u + 1];
-    if (j1 - j0 > a.H) continue;
-    float4 pu[VPL], acc[VPL];
-#pragma unroll
-    for (int v = 0; v < VPL; ++v) {
-      pu[v] = own_row(i, v);
-      acc[v] = f4_zero();
-    }
-    gather_range<LPR, VPL, WEIGHTED, true, RUB>(a, src_rows, gl, gm, 0, nvec, pu, j0, j1, acc, on);
-#pragma unroll
-    for (int v = 0; v < VPL; ++v) {
-      const int q = gl + LPR * v;
-      if (q >= nvec) continue;
-      float4 o;
-      o.x = fmaf(a.eps, pu[v].x, acc[v].x);
-      o.y = fmaf(a.eps, pu[v].y, acc[v].y);
-      o.z = fmaf(a.eps, pu[v].z, acc[v].z);
-      o.w = fmaf(a.eps, pu[v].w, acc[v].w);
-      emit(i, v, pu[v], o);
-    }
+    const int mine = nrows > gi ? (nrows - gi + GPB - 1) / GPB : 0;
+    walk_rows<LPR, RUB<LPR>, WEIGHTED, true>(
+        a, srcq, gl, gm, slots, mine, lane_on,
+        [&](int k, uint32_t& j, int& len, uint32_t& u) {
+          u = (uint32_t)(r0 + (gi + k * GPB) * rstep);
+          uint32_t n;
+          row_slots(a.row_ptr, u, j, n);
+          len = n > (uint32_t)a.H ? -1 : (int)n;
+        },
+        own_quad,
+        [&](int k, uint32_t u, Quad pu, Quad acc) {
+          if (valid)
+            emit(gi + k * GPB, (int64_t)u, v, unquad(pu), unquad(apply_quad(a.eps, pu, acc)));
+        });
   }
 }
 
@@ -390,11 +486,12 @@ __global__ void __launch_bounds__(PT, 1) k_cg_resident(ResArgs ra) {
   float* aps = rs + (size_t)ra.rb * ld;                // [rb][ld]  Ap of own rows
   float* ps = aps + (size_t)ra.rb * ld;                // [rb][ld]  p of own rows (PS only)
   float2* sbuf = reinterpret_cast<float2*>(PS ? ps + (size_t)ra.rb * ld : ps);  // [ld]
-  // one region, used as the heavy-row slices [GPB][ld] in the operator and as the reduction
-  // scratch [PWARPS][PCH] = 2 * PT float pairs after it; then the local heavy-row list [rb]
+  // one region, used as the heavy-row slices [hrows][PT] in the operator and as the reduction
+  // scratch [PWARPS][PCH] = 2 * PT float pairs after it; then the heavy-row list [rb] of the rows
+  // the block gathers
   float* comb = reinterpret_cast<float*>(sbuf + ld);
   float2* scratch = sbuf + ld;
-  int* hv = reinterpret_cast<int*>(comb + resident_shared_floats(ld));
+  int* hv = reinterpret_cast<int*>(comb + resident_shared_floats(ra.hrows));
   // block partials, one region per reduction kind so that no block overwrites partials another
   // block may still be summing: [G][ld] each
   float2* part_pap = a.cr.part1;
@@ -413,13 +510,33 @@ __global__ void __launch_bounds__(PT, 1) k_cg_resident(ResArgs ra) {
   __shared__ __align__(16) int s_active[RMAXLD];
   __shared__ int s_iters[RMAXLD], s_conv[RMAXLD];
   __shared__ int s_nh, s_wcnt[PWARPS];
+  __shared__ unsigned s_most;
+  __shared__ Slots<RUB<LPR>, WEIGHTED> slots[GPB];
 
-  // ---- the block's rows heavier than a.H, ascending
-  if (threadIdx.x == 0) s_nh = 0;
+  // ---- which rows the block gathers in A: its own, or dealt ones where the own ranges are so
+  // uneven that the largest would cost more than 4 us an iteration over the mean.  A gathered
+  // 128-byte line costs about 1 ns of an SM (the gathers run at 13 to 20 TB/s over 152 SMs): 4,000
+  // lines, where handing Ap over through L2 costs under a microsecond.  Every block finds the same.
+  if (threadIdx.x == 0) {
+    s_nh = 0;
+    s_most = 0;
+  }
   __syncthreads();
-  for (int base = 0; base < nrows; base += PT) {
+  for (int b = threadIdx.x; b < G; b += PT) {
+    const int64_t lo = min((int64_t)a.n, (int64_t)b * ra.rb), hi = min((int64_t)a.n, lo + ra.rb);
+    atomicMax(&s_most, (unsigned)(a.row_ptr[hi] - a.row_ptr[lo]));
+  }
+  __syncthreads();
+  const int64_t excess = (int64_t)s_most - a.row_ptr[a.n] / G;
+  const bool deal = excess * ((ld + 31) / 32) > 4000;
+  const int64_t g0 = deal ? blockIdx.x : r0, gstep = deal ? G : 1;  // rows g0 + i gstep, i < grows
+  const int grows = !deal ? nrows : a.n > g0 ? (int)((a.n - g0 + G - 1) / G) : 0;
+
+  // ---- those of them heavier than a.H, ascending
+  for (int base = 0; base < grows; base += PT) {
     const int i = base + threadIdx.x;
-    const bool heavy = i < nrows && a.row_ptr[r0 + i + 1] - a.row_ptr[r0 + i] > a.H;
+    const bool heavy =
+        i < grows && a.row_ptr[g0 + i * gstep + 1] - a.row_ptr[g0 + i * gstep] > a.H;
     const unsigned bal = __ballot_sync(0xffffffffu, heavy);
     if (lane == 0) s_wcnt[warp] = __popc(bal);
     __syncthreads();
@@ -539,9 +656,18 @@ __global__ void __launch_bounds__(PT, 1) k_cg_resident(ResArgs ra) {
 #pragma unroll
       for (int t = 0; t < 4; ++t) dot[v][t] = make_float2(0.f, 0.f);
     block_apply<LPR, VPL, WEIGHTED>(
-        a, a.P, PS ? ps : nullptr, r0, nrows, hv, nh, comb, gl, gi, gm, on,
-        [&](int i, int v, float4 pu, float4 o) {
-          reinterpret_cast<float4*>(aps + (size_t)i * ld)[gl + LPR * v] = o;
+        a, a.P, g0, gstep, grows, hv, nh, ra.hrows, comb, slots[gi], gl, gi, gm, on,
+        [&](int64_t u, int v) {
+          const int q = gl + LPR * v;
+          return PS && !deal ? reinterpret_cast<const float4*>(ps + (size_t)(u - r0) * ld)[q]
+                             : ldcg_f4(a.P + (size_t)u * ld + 4 * q);
+        },
+        [&](int i, int64_t u, int v, float4 pu, float4 o) {
+          const int q = gl + LPR * v;
+          if (deal)
+            *reinterpret_cast<float4*>(a.AP + (size_t)u * ld + 4 * q) = o;
+          else
+            reinterpret_cast<float4*>(aps + (size_t)i * ld)[q] = o;
           dot[v][0] = df_fma(dot[v][0], pu.x, o.x);
           dot[v][1] = df_fma(dot[v][1], pu.y, o.y);
           dot[v][2] = df_fma(dot[v][2], pu.z, o.z);
@@ -578,7 +704,7 @@ __global__ void __launch_bounds__(PT, 1) k_cg_resident(ResArgs ra) {
 #pragma unroll
       for (int t = 0; t < 4; ++t) dz[v][t] = make_float2(0.f, 0.f);
     for (int i0 = gi; i0 < nrows; i0 += NU * GPB) {
-      float4 p[NU][VPL], x[NU][VPL];
+      float4 p[NU][VPL], x[NU][VPL], ap[NU][VPL];
       float di[NU];
 #pragma unroll
       for (int k = 0; k < NU; ++k)
@@ -592,6 +718,8 @@ __global__ void __launch_bounds__(PT, 1) k_cg_resident(ResArgs ra) {
             const size_t o = (size_t)(r0 + i) * ld + 4 * q;
             p[k][v] = PS ? reinterpret_cast<const float4*>(ps + (size_t)i * ld)[q] : ldcg_f4(a.P + o);
             x[k][v] = *reinterpret_cast<const float4*>(va.X + o);
+            ap[k][v] = deal ? ldcg_f4(a.AP + o)
+                            : reinterpret_cast<const float4*>(aps + (size_t)i * ld)[q];
           }
         }
 #pragma unroll
@@ -601,15 +729,15 @@ __global__ void __launch_bounds__(PT, 1) k_cg_resident(ResArgs ra) {
           const int i = i0 + k * GPB, q = gl + LPR * v;
           if (i >= nrows || q >= nvec || !((on >> v) & 1u)) continue;
           float4 xx = x[k][v], r = reinterpret_cast<const float4*>(rs + (size_t)i * ld)[q];
-          const float4 pp = p[k][v], ap = reinterpret_cast<const float4*>(aps + (size_t)i * ld)[q];
+          const float4 pp = p[k][v];
           xx.x = fmaf(al[v].x, pp.x, xx.x);
           xx.y = fmaf(al[v].y, pp.y, xx.y);
           xx.z = fmaf(al[v].z, pp.z, xx.z);
           xx.w = fmaf(al[v].w, pp.w, xx.w);
-          r.x = fmaf(-al[v].x, ap.x, r.x);
-          r.y = fmaf(-al[v].y, ap.y, r.y);
-          r.z = fmaf(-al[v].z, ap.z, r.z);
-          r.w = fmaf(-al[v].w, ap.w, r.w);
+          r.x = fmaf(-al[v].x, ap[k][v].x, r.x);
+          r.y = fmaf(-al[v].y, ap[k][v].y, r.y);
+          r.z = fmaf(-al[v].z, ap[k][v].z, r.z);
+          r.w = fmaf(-al[v].w, ap[k][v].w, r.w);
           *reinterpret_cast<float4*>(va.X + (size_t)(r0 + i) * ld + 4 * q) = xx;
           reinterpret_cast<float4*>(rs + (size_t)i * ld)[q] = r;
           dot[v][0] = df_fma(dot[v][0], r.x, r.x);
@@ -722,10 +850,11 @@ __global__ void __launch_bounds__(PT, 1) k_cg_resident(ResArgs ra) {
 #pragma unroll
     for (int t = 0; t < 4; ++t) dot[v][t] = make_float2(0.f, 0.f);
   block_apply<LPR, VPL, WEIGHTED>(
-      a, va.X, nullptr, r0, nrows, hv, nh, comb, gl, gi, gm, ~0u,
-      [&](int i, int v, float4, float4 o) {
+      a, va.X, g0, gstep, grows, hv, nh, ra.hrows, comb, slots[gi], gl, gi, gm, ~0u,
+      [&](int64_t u, int v) { return ldcg_f4(va.X + (size_t)u * ld + 4 * (gl + LPR * v)); },
+      [&](int, int64_t u, int v, float4, float4 o) {
         const int q = gl + LPR * v, cb = 4 * q;
-        const float4 y = ld_f4(a.Y + (size_t)(r0 + i) * ld + 4 * q);
+        const float4 y = ld_f4(a.Y + (size_t)u * ld + 4 * q);
         const float rx = cb + 0 < a.kc ? y.x - o.x : 0.f;
         const float ry = cb + 1 < a.kc ? y.y - o.y : 0.f;
         const float rz = cb + 2 < a.kc ? y.z - o.z : 0.f;
