@@ -420,6 +420,7 @@ __device__ __forceinline__ bool aborted(const unsigned* abort) {
 // internal entry points shared between translation units
 // ------------------------------------------------------------------------------------------------
 erc_status check_graph(const erc_graph* g);
+constexpr unsigned LOOKBACK_SPINS = 1u << 22;  // polls of a predecessor tile before giving up
 size_t scan_temp_bytes(int64_t n);
 // exclusive scan of int64 `in` (or of the 0/1 flags in `flags` when `in` is null) into `out`;
 // `total` (device, may be null) receives the sum.  `abort` (device, required) is the call's abort
@@ -427,11 +428,22 @@ size_t scan_temp_bytes(int64_t n);
 // gives up (the output is then incomplete; every entry stays within [0, the true value]).
 erc_status exclusive_scan_i64(const int64_t* in, const uint8_t* flags, int64_t* out, int64_t n,
                               int64_t* total, void* tmp, cudaStream_t s, unsigned* abort);
-size_t radix_sort_temp_bytes(int64_t n);
-// stable LSD radix sort of (key, value) pairs on the low `bits` key bits; the result is in
-// keys/vals (the *_alt buffers are scratch of the same size).  `abort` as for the scan: once it
-// is set no further pass runs and the result is undefined.
-erc_status radix_sort_pairs(uint64_t* keys, uint32_t* vals, uint64_t* keys_alt, uint32_t* vals_alt,
-                            int64_t n, int bits, void* tmp, cudaStream_t s, unsigned* abort);
+// Passes of a stable LSD radix sort of (key, value) pairs by 8-bit digits.  The caller zeroes the
+// temporary storage once (radix_sort_begin) and numbers its passes 0, 1, ..., also across several
+// sorts that share it; n_max bounds every one of them.  A pass sorts by key bits [shift, shift +
+// 8) the first min(n_max, *n) pairs (all n_max when n, a device pointer, is null); vals may be null.
+// counts[RS_RADIX] (device) holds how many of those keys have each digit.  radix_sort_open raises the
+// kernel's shared-memory limit on the current device: once before the passes are enqueued or
+// captured.  `abort` as for the scan: once it is set no further pass runs and the result is
+// undefined.
+constexpr int RS_BITS = 8;
+constexpr int RS_MAX_PASSES = 16;
+size_t radix_sort_temp_bytes(int64_t n_max);
+erc_status radix_sort_open();
+erc_status radix_sort_begin(int64_t n_max, void* tmp, cudaStream_t s);
+erc_status radix_sort_pass(const uint64_t* keys, const uint32_t* vals, uint64_t* keys_out,
+                           uint32_t* vals_out, int64_t n_max, const int64_t* n, int shift, int pass,
+                           const unsigned long long* counts, void* tmp, cudaStream_t s,
+                           unsigned* abort);
 
 }  // namespace erc

@@ -1,5 +1,6 @@
-// sort_scan.cu -- device-wide exclusive scan (int64) and stable LSD radix sort of (u64 key, u32 value)
-// pairs.  Used once per graph by the Laplacian build (§3.1.1); both are deterministic.
+// sort_scan.cu -- device-wide exclusive scan (int64) for the samplers (§3.2) and the passes of a
+// stable LSD radix sort of (u64 key, u32 value) pairs for the Laplacian build (§3.1.1); both are
+// deterministic.
 #include "erc_internal.cuh"
 
 namespace erc {
@@ -61,8 +62,6 @@ __device__ __forceinline__ int64_t block_exclusive_scan(int64_t v, int64_t* bloc
 // prefix of zero, so its output stays within [0, the true prefix].  A block that starts after the
 // abort word is set takes no ticket and does nothing: no tile ever waits on a tile that no block
 // has claimed.
-constexpr unsigned LOOKBACK_SPINS = 1u << 22;
-
 template <class Load>
 __global__ void __launch_bounds__(SCAN_THREADS)
     k_scan_onepass(Load in, int64_t n, unsigned long long* status, unsigned* ticket, int64_t* out,
@@ -175,126 +174,163 @@ erc_status scan_impl(Load in, int64_t n, int64_t* out, int64_t* total, int64_t* 
 }
 
 // ------------------------------------------------------------------------------------------------
-// radix sort: RB-bit digits (8, or 10 while the per-tile count table stays small: 3 passes instead
-// of 4 for the 30-bit keys of a 20k-node graph), tiles of 2048 keys; a block's tile is split into
-// 8 warp sub-tiles in warp-striped order so that (warp, step, lane) order equals key order, which
-// makes the ranks stable.
+// Stable LSD radix sort of (u64 key, u32 value) pairs, one kernel per 8-bit digit (the digit counts
+// of every pass come from the kernel that wrote the keys): a tile ranks its keys, publishes its
+// digit counts, learns the counts of the tiles before it by decoupled look-back (as in the scan
+// above, one digit per thread) and writes its keys.  What bounds a pass is HBM: 12 bytes read and
+// written per pair.  The tile is therefore brought into digit order in shared memory first, so
+// that a digit's keys leave as one run (16 keys, 128 bytes on average) instead of one 8-byte and
+// one 4-byte store each (the three kernels per pass it replaces -- count, scan, scatter straight
+// from registers -- took 3.8 ms for 131M pairs).
+// A block's tile is split into warp sub-tiles in warp-striped order so that (warp, step, lane)
+// order equals key order, which makes the ranks stable.
+// A status word holds value << 16 | pass << 2 | flag: no pass needs its status cleared.
 // ------------------------------------------------------------------------------------------------
-constexpr int RS_THREADS = 256;
+constexpr int RS_THREADS = 256;  // one digit per thread
 constexpr int RS_WARPS = RS_THREADS / 32;
-constexpr int RS_IPT = 8;
+constexpr int RS_IPT = 16;
 constexpr int RS_TILE = RS_THREADS * RS_IPT;
-constexpr int64_t RS_WIDE_MAX_TILES = 4096;  // 10-bit digits up to 8M keys
+constexpr int RS_RADIX = 1 << RS_BITS;
+static_assert(RS_RADIX == RS_THREADS, "one digit per thread");
 
-inline int radix_bits(int64_t n) { return (n + RS_TILE - 1) / RS_TILE <= RS_WIDE_MAX_TILES ? 10 : 8; }
+struct SortShared {
+  uint64_t key[RS_TILE];
+  uint32_t val[RS_TILE];
+  unsigned whist[RS_WARPS][RS_RADIX];
+  unsigned local[RS_RADIX];  // first slot of a digit's keys in the tile
+  int64_t dest[RS_RADIX];    // where the digit's keys go, less `local`
+  unsigned wsum[RS_WARPS];
+  unsigned tile;
+};
 
-template <int RB>
+template <bool VALS>
 __global__ void __launch_bounds__(RS_THREADS)
-    k_radix_hist(const uint64_t* keys, int64_t n, int shift, int64_t* counts, int64_t nb,
-                 const unsigned* abort) {
-  constexpr unsigned RADIX = 1u << RB;
-  __shared__ unsigned hist[RADIX];
-  if (aborted(abort)) return;
-  for (unsigned d = threadIdx.x; d < RADIX; d += RS_THREADS) hist[d] = 0;
+    k_radix_pass(const uint64_t* __restrict__ keys, const uint32_t* __restrict__ vals,
+                 uint64_t* __restrict__ keys_out, uint32_t* __restrict__ vals_out, int64_t n_max,
+                 const int64_t* __restrict__ n_ptr, int shift, int pass,
+                 const unsigned long long* __restrict__ counts, unsigned long long* status,
+                 unsigned* ticket, unsigned* abort, unsigned spin_limit) {
+  extern __shared__ __align__(16) unsigned char sort_smem[];
+  SortShared& sh = *reinterpret_cast<SortShared*>(sort_smem);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (tid == 0) sh.tile = aborted(abort) ? 0xffffffffu : atomicAdd(ticket, 1u);
+  for (int d = lane; d < RS_RADIX; d += 32) sh.whist[warp][d] = 0;
   __syncthreads();
-  const int64_t base = (int64_t)blockIdx.x * RS_TILE;
-#pragma unroll
-  for (int j = 0; j < RS_IPT; ++j) {
-    int64_t i = base + j * RS_THREADS + threadIdx.x;
-    if (i < n) atomicAdd(&hist[(unsigned)(keys[i] >> shift) & (RADIX - 1)], 1u);
-  }
-  __syncthreads();
-  for (unsigned d = threadIdx.x; d < RADIX; d += RS_THREADS)
-    counts[(int64_t)d * nb + blockIdx.x] = hist[d];
-}
+  if (sh.tile == 0xffffffffu) return;
+  const int64_t n = n_ptr ? min(n_max, *n_ptr) : n_max;
+  const int64_t t = sh.tile, tile0 = t * RS_TILE;
+  if (tile0 >= n) return;  // nobody waits on a tile past the end
+  const int count = (int)min((int64_t)RS_TILE, n - tile0);
 
-template <int RB>
-__global__ void __launch_bounds__(RS_THREADS)
-    k_radix_scatter(const uint64_t* __restrict__ keys, const uint32_t* __restrict__ vals,
-                    uint64_t* __restrict__ keys_out, uint32_t* __restrict__ vals_out, int64_t n,
-                    int shift, const int64_t* __restrict__ offsets, int64_t nb,
-                    const unsigned* abort) {
-  constexpr unsigned RADIX = 1u << RB;
-  __shared__ unsigned whist[RS_WARPS][RADIX];
-  __shared__ int64_t boff[RADIX];
-  if (aborted(abort)) return;  // the offsets of an unfinished scan are not used
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (unsigned d = threadIdx.x; d < RADIX * RS_WARPS; d += RS_THREADS) (&whist[0][0])[d] = 0;
-  for (unsigned d = threadIdx.x; d < RADIX; d += RS_THREADS)
-    boff[d] = offsets[(int64_t)d * nb + blockIdx.x];
-  __syncthreads();
-  const int64_t base = (int64_t)blockIdx.x * RS_TILE + (int64_t)warp * 32 * RS_IPT;
+  // ---- keys in warp-striped order, ranked among the warp's equal digits
+  const int sub = warp * 32 * RS_IPT;
   const unsigned lt_mask = (1u << lane) - 1u;
   uint64_t k[RS_IPT];
-  uint32_t v[RS_IPT];
-  unsigned rank[RS_IPT];
-  unsigned dig[RS_IPT];
+  uint32_t v[VALS ? RS_IPT : 1];
+  unsigned short rank[RS_IPT];
 #pragma unroll
   for (int j = 0; j < RS_IPT; ++j) {
-    int64_t i = base + j * 32 + lane;
-    bool ok = i < n;
-    k[j] = ok ? keys[i] : 0;
-    v[j] = ok ? vals[i] : 0;
-    unsigned d = ok ? ((unsigned)(k[j] >> shift) & (RADIX - 1)) : RADIX;
-    dig[j] = d;
-    unsigned peers = __match_any_sync(0xffffffffu, d);
-    unsigned before = 0;
-    if (ok) before = whist[warp][d];
-    __syncwarp();
-    if (ok && lane == __ffs(peers) - 1) whist[warp][d] = before + __popc(peers);
-    __syncwarp();
-    rank[j] = before + __popc(peers & lt_mask);
+    const int i = sub + j * 32 + lane;
+    k[j] = i < count ? keys[tile0 + i] : 0;
+    if (VALS) v[j] = i < count ? vals[tile0 + i] : 0;
   }
-  __syncthreads();
-  // exclusive prefix over warps per digit, plus the block's global offset for the digit
-  for (unsigned d = threadIdx.x; d < RADIX; d += RS_THREADS) {
-    unsigned run = 0;
-    for (int w = 0; w < RS_WARPS; ++w) {
-      unsigned t = whist[w][d];
-      whist[w][d] = run;
-      run += t;
-    }
-  }
-  __syncthreads();
 #pragma unroll
   for (int j = 0; j < RS_IPT; ++j) {
-    if (dig[j] < RADIX) {
-      int64_t dst = boff[dig[j]] + whist[warp][dig[j]] + rank[j];
-      keys_out[dst] = k[j];
-      vals_out[dst] = v[j];
-    }
+    const bool ok = sub + j * 32 + lane < count;
+    const unsigned d = ok ? (unsigned)(k[j] >> shift) & (RS_RADIX - 1) : RS_RADIX;
+    const unsigned peers = __match_any_sync(0xffffffffu, d);
+    const unsigned before = ok ? sh.whist[warp][d] : 0;
+    __syncwarp();
+    if (ok && lane == __ffs(peers) - 1) sh.whist[warp][d] = before + __popc(peers);
+    __syncwarp();
+    rank[j] = (unsigned short)(before + __popc(peers & lt_mask));
   }
-}
+  __syncthreads();
 
-template <int RB>
-erc_status radix_passes(uint64_t* keys, uint32_t* vals, uint64_t* keys_alt, uint32_t* vals_alt,
-                        int64_t n, int bits, void* tmp, cudaStream_t s, unsigned* abort) {
-  const int64_t nb = (n + RS_TILE - 1) / RS_TILE;
-  const size_t cnt = (size_t)nb << RB;
-  char* t = static_cast<char*>(tmp);
-  int64_t* counts = reinterpret_cast<int64_t*>(t);
-  int64_t* offs = reinterpret_cast<int64_t*>(t + ((cnt * sizeof(int64_t) + 255) & ~size_t(255)));
-  void* scan_tmp = t + 2 * ((cnt * sizeof(int64_t) + 255) & ~size_t(255));
-  uint64_t *ka = keys, *kb = keys_alt;
-  uint32_t *va = vals, *vb = vals_alt;
-  int passes = 0;
-  for (int shift = 0; shift < bits; shift += RB, ++passes) {
-    k_radix_hist<RB><<<(unsigned)nb, RS_THREADS, 0, s>>>(ka, n, shift, counts, nb, abort);
-    count_launches(1);
-    ERC_CUDA(cudaGetLastError());
-    ERC_TRY(exclusive_scan_i64(counts, nullptr, offs, (int64_t)cnt, nullptr, scan_tmp, s, abort));
-    k_radix_scatter<RB><<<(unsigned)nb, RS_THREADS, 0, s>>>(ka, va, kb, vb, n, shift, offs, nb,
-                                                            abort);
-    count_launches(1);
-    ERC_CUDA(cudaGetLastError());
-    uint64_t* tk = ka; ka = kb; kb = tk;
-    uint32_t* tv = va; va = vb; vb = tv;
+  // ---- digit tid: its keys in this tile, published; its first slot in the tile
+  unsigned mine = 0;
+#pragma unroll
+  for (int w = 0; w < RS_WARPS; ++w) {
+    const unsigned c = sh.whist[w][tid];
+    sh.whist[w][tid] = mine;
+    mine += c;
   }
-  if (passes & 1) {  // the result sits in the alternate buffers: copy it back
-    ERC_CUDA(cudaMemcpyAsync(keys, ka, (size_t)n * sizeof(uint64_t), cudaMemcpyDeviceToDevice, s));
-    ERC_CUDA(cudaMemcpyAsync(vals, va, (size_t)n * sizeof(uint32_t), cudaMemcpyDeviceToDevice, s));
+  const unsigned long long tag = (unsigned long long)(pass + 1) << 2;
+  volatile unsigned long long* st = status;
+  st[t * RS_RADIX + tid] = (unsigned long long)mine << 16 | tag | (t == 0 ? 2ull : 1ull);
+  unsigned inc = mine;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned x = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += x;
   }
-  return ERC_OK;
+  // the digit's first key over all tiles: the counts of the smaller digits
+  unsigned long long base = counts[tid], binc = base;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned long long x = __shfl_up_sync(0xffffffffu, binc, o);
+    if (lane >= o) binc += x;
+  }
+  __shared__ unsigned long long wbase[RS_WARPS];
+  if (lane == 31) {
+    sh.wsum[warp] = inc;
+    wbase[warp] = binc;
+  }
+  __syncthreads();
+  unsigned local = inc - mine;
+  unsigned long long dest = binc - base;
+  for (int w = 0; w < warp; ++w) {
+    local += sh.wsum[w];
+    dest += wbase[w];
+  }
+  sh.local[tid] = local;
+
+  // ---- the keys into digit order (overlaps the wait for the tiles before)
+  __syncthreads();
+#pragma unroll
+  for (int j = 0; j < RS_IPT; ++j) {
+    if (sub + j * 32 + lane >= count) continue;
+    const unsigned d = (unsigned)(k[j] >> shift) & (RS_RADIX - 1);
+    const unsigned at = sh.local[d] + sh.whist[warp][d] + rank[j];
+    sh.key[at] = k[j];
+    if (VALS) sh.val[at] = v[j];
+  }
+
+  // ---- digit tid in the tiles before this one, eight status words a trip
+  if (t > 0) {
+    unsigned long long before = 0;
+    bool done = false;
+    for (int64_t q = t - 1; !done; q -= 8) {
+      unsigned long long w[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) w[i] = q - i >= 0 ? st[(q - i) * RS_RADIX + tid] : 0;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        if (done) break;
+        unsigned spins = 0;
+        while ((w[i] & 0xfffcull) != tag) {  // not published yet
+          if (++spins > spin_limit || aborted(abort)) {  // bounded: record it and take zero
+            atomicOr(abort, 1u);
+            w[i] = tag | 2ull;
+            break;
+          }
+          w[i] = st[(q - i) * RS_RADIX + tid];
+        }
+        before += w[i] >> 16;
+        done = (w[i] & 3ull) == 2ull;  // tile 0 always is
+      }
+    }
+    st[t * RS_RADIX + tid] = (before + mine) << 16 | tag | 2ull;
+    dest += before;
+  }
+  sh.dest[tid] = (int64_t)dest - local;
+  __syncthreads();
+  for (int i = tid; i < count; i += RS_THREADS) {
+    const uint64_t key = sh.key[i];
+    const int64_t at = sh.dest[(unsigned)(key >> shift) & (RS_RADIX - 1)] + i;
+    keys_out[at] = key;
+    if (VALS) vals_out[at] = sh.val[i];
+  }
 }
 
 }  // namespace
@@ -309,18 +345,48 @@ erc_status exclusive_scan_i64(const int64_t* in, const uint8_t* flags, int64_t* 
   return scan_impl(LoadFlag{flags}, n, out, total, static_cast<int64_t*>(tmp), s, abort);
 }
 
+inline int64_t sort_tiles(int64_t n) { return (n + RS_TILE - 1) / RS_TILE; }
+
+// tmp: [status: tiles x RS_RADIX][tickets: RS_MAX_PASSES]
 size_t radix_sort_temp_bytes(int64_t n) {
-  const int64_t nb = (n + RS_TILE - 1) / RS_TILE;
-  const size_t cnt = (size_t)nb << radix_bits(n);
-  return 2 * ((cnt * sizeof(int64_t) + 255) & ~size_t(255)) + scan_temp_bytes((int64_t)cnt);
+  return (size_t)sort_tiles(n > 0 ? n : 1) * RS_RADIX * sizeof(unsigned long long) +
+         RS_MAX_PASSES * sizeof(unsigned);
 }
 
-erc_status radix_sort_pairs(uint64_t* keys, uint32_t* vals, uint64_t* keys_alt, uint32_t* vals_alt,
-                            int64_t n, int bits, void* tmp, cudaStream_t s, unsigned* abort) {
-  if (n <= 1) return ERC_OK;
-  if (radix_bits(n) == 10)
-    return radix_passes<10>(keys, vals, keys_alt, vals_alt, n, bits, tmp, s, abort);
-  return radix_passes<8>(keys, vals, keys_alt, vals_alt, n, bits, tmp, s, abort);
+erc_status radix_sort_begin(int64_t n, void* tmp, cudaStream_t s) {
+  ERC_CUDA(cudaMemsetAsync(tmp, 0, radix_sort_temp_bytes(n), s));
+  return ERC_OK;
+}
+
+erc_status radix_sort_open() {
+  const int bytes = (int)sizeof(SortShared);
+  ERC_CUDA(cudaFuncSetAttribute((const void*)k_radix_pass<true>,
+                                cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+  ERC_CUDA(cudaFuncSetAttribute((const void*)k_radix_pass<false>,
+                                cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+  return ERC_OK;
+}
+
+erc_status radix_sort_pass(const uint64_t* keys, const uint32_t* vals, uint64_t* keys_out,
+                           uint32_t* vals_out, int64_t n_max, const int64_t* n, int shift, int pass,
+                           const unsigned long long* counts, void* tmp, cudaStream_t s,
+                           unsigned* abort) {
+  if (n_max <= 0) return ERC_OK;
+  unsigned long long* status = static_cast<unsigned long long*>(tmp);
+  unsigned* tickets = reinterpret_cast<unsigned*>(status + sort_tiles(n_max) * RS_RADIX);
+  const unsigned grid = (unsigned)sort_tiles(n_max);
+  const unsigned limit = wait_limit(LOOKBACK_SPINS);
+  if (vals)
+    k_radix_pass<true><<<grid, RS_THREADS, sizeof(SortShared), s>>>(
+        keys, vals, keys_out, vals_out, n_max, n, shift, pass, counts, status, tickets + pass,
+        abort, limit);
+  else
+    k_radix_pass<false><<<grid, RS_THREADS, sizeof(SortShared), s>>>(
+        keys, nullptr, keys_out, nullptr, n_max, n, shift, pass, counts, status, tickets + pass,
+        abort, limit);
+  count_launches(1);
+  ERC_CUDA(cudaGetLastError());
+  return ERC_OK;
 }
 
 }  // namespace erc
