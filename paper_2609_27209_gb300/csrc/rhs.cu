@@ -10,78 +10,85 @@ namespace erc {
 namespace {
 
 // Row u of Y: the LPR lanes of a group walk u's CSR slots LPR at a time.  Lane l generates the
-// Philox blocks of slot jb + l (one per 128-column block its group covers) and the slot's signed
-// coefficient; the slots are then applied in CSR order, each lane taking from the generating
-// lane, by shuffles, the word that holds its four columns' sign bits.
+// Philox words of slot jb + l (one block of four words per 128 columns that the group covers) and
+// leaves them in shared memory with the slot's coefficient; the slots are then applied in CSR
+// order, each lane reading the one word that holds its four columns' signs.  The orientation sigma
+// goes into the words (all signs of a slot flipped), and a sign is applied by moving its bit to the
+// coefficient's sign bit, two columns an addition.
+//
+// What bounds it is instruction issue: each of the 2m slots costs a lane two shared loads and a
+// dozen operations (passing the words by shuffles, four a slot and the selection of one of them,
+// took about 28).  2.45M nodes, 64.3M edges, 128 columns: 2.77 ms, 6.71 ms with the shuffles.
 template <int LPR, int VPL, bool WEIGHTED>
 __global__ void __launch_bounds__(256)
     k_jl_rhs(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
              const float* __restrict__ val, const int32_t* __restrict__ csr_eid, int32_t n,
              uint2 key, float inv_sqrt_k, int32_t c0, int32_t kc, int32_t ld, float* __restrict__ Y) {
-  constexpr int NBM = VPL + 1;  // 128-column Philox blocks a group's columns can span
-  const int gl = threadIdx.x & (LPR - 1);
+  constexpr int NB = (4 * LPR * VPL + 127) / 128 + 1;  // 128-column Philox blocks a group can span
+  constexpr int GPB = 256 / LPR;
+  // a slot's words; groups are padded apart so that they meet in different banks
+  __shared__ __align__(16) uint32_t s_word[GPB][LPR * 4 * NB + 4];
+  __shared__ float s_coef[WEIGHTED ? GPB : 1][WEIGHTED ? LPR : 1];
+  const int gl = threadIdx.x & (LPR - 1), gi = threadIdx.x / LPR;
   const unsigned gm = group_mask<LPR>();
-  const int groups_per_block = blockDim.x / LPR;
-  const int64_t ngroups = (int64_t)gridDim.x * groups_per_block;
+  const int64_t ngroups = (int64_t)gridDim.x * GPB;
   const int nvec = ld >> 2;
   const int g0 = c0 >> 7;
   const int nb = ((c0 + 4 * (nvec - 1)) >> 7) - g0 + 1;
-  int blk[VPL], wsel[VPL], sh[VPL];
-  bool on[VPL];
+  int at[VPL], sh[VPL];  // the lane's word among a slot's 4 NB, and the shift of its columns' bits
 #pragma unroll
   for (int v = 0; v < VPL; ++v) {
-    const int q = gl + LPR * v;
+    const int q = min(gl + LPR * v, nvec - 1);
     const int c = c0 + 4 * q;  // c0 % 4 == 0: the four columns share one word
-    on[v] = q < nvec && 4 * q < kc;
-    blk[v] = (c >> 7) - g0;
-    wsel[v] = (c >> 5) & 3;
-    sh[v] = c & 31;
+    at[v] = (c >> 5) - 4 * g0;
+    sh[v] = 28 - (c & 31);  // the column's bit 0 to bit 28, and so on to bit 31
   }
-  for (int64_t u = (int64_t)blockIdx.x * groups_per_block + threadIdx.x / LPR; u < n;
-       u += ngroups) {
+  for (int64_t u = (int64_t)blockIdx.x * GPB + gi; u < n; u += ngroups) {
     float4 acc[VPL];
 #pragma unroll
     for (int v = 0; v < VPL; ++v) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
     const int64_t j0 = row_ptr[u], j1 = row_ptr[u + 1];
+    // the next slots' ids are loaded before the present ones are applied
+    uint32_t e = 0;
+    int32_t other = 0;
+    float w = 0.f;
+    auto fetch = [&](int64_t j) {
+      if (j >= j1) return;
+      e = (uint32_t)__ldg(csr_eid + j);
+      other = __ldg(col + j);
+      if (WEIGHTED) w = __ldg(val + j);
+    };
+    fetch(j0 + gl);
     for (int64_t jb = j0; jb < j1; jb += LPR) {
-      const int64_t j = jb + gl;
-      float coef = 0.f;
-      uint4 w[NBM];
+      if (jb + gl < j1) {
+        const uint32_t flip = other < u ? ~0u : 0u;  // u is the larger endpoint: row e is e_nb - e_u
 #pragma unroll
-      for (int b = 0; b < NBM; ++b) w[b] = make_uint4(0u, 0u, 0u, 0u);
-      if (j < j1) {
-        const uint32_t e = (uint32_t)csr_eid[j];
-        coef = WEIGHTED ? sqrtf(val[j]) * inv_sqrt_k : inv_sqrt_k;
-        if (col[j] < u) coef = -coef;  // u is the larger endpoint: row e of B is e_nb - e_u
-#pragma unroll
-        for (int b = 0; b < NBM; ++b)
-          if (b < nb) w[b] = philox4x32_10(make_uint4((uint32_t)(g0 + b), 0u, e, 0u), key);
-      }
-      const int cnt = (int)min((int64_t)LPR, j1 - jb);
-      for (int k = 0; k < cnt; ++k) {
-        const float cf = __shfl_sync(gm, coef, k, LPR);
-        uint32_t word[VPL];
-#pragma unroll
-        for (int v = 0; v < VPL; ++v) word[v] = 0u;
-#pragma unroll
-        for (int b = 0; b < NBM; ++b) {
+        for (int b = 0; b < NB; ++b) {
           if (b >= nb) break;
-          const uint32_t x = __shfl_sync(gm, w[b].x, k, LPR), y = __shfl_sync(gm, w[b].y, k, LPR);
-          const uint32_t z = __shfl_sync(gm, w[b].z, k, LPR), t = __shfl_sync(gm, w[b].w, k, LPR);
-#pragma unroll
-          for (int v = 0; v < VPL; ++v)
-            if (blk[v] == b) word[v] = wsel[v] == 0 ? x : wsel[v] == 1 ? y : wsel[v] == 2 ? z : t;
+          const uint4 x = philox4x32_10(make_uint4((uint32_t)(g0 + b), 0u, e, 0u), key);
+          *reinterpret_cast<uint4*>(s_word[gi] + gl * 4 * NB + 4 * b) =
+              make_uint4(x.x ^ flip, x.y ^ flip, x.z ^ flip, x.w ^ flip);
         }
+        if (WEIGHTED) s_coef[gi][gl] = sqrtf(w) * inv_sqrt_k;
+      }
+      fetch(jb + LPR + gl);
+      __syncwarp(gm);
+      const int cnt = (int)min((int64_t)LPR, j1 - jb);
+#pragma unroll 4
+      for (int k = 0; k < cnt; ++k) {
+        const uint32_t cf = __float_as_uint(WEIGHTED ? s_coef[WEIGHTED ? gi : 0][WEIGHTED ? k : 0]
+                                                     : inv_sqrt_k);
 #pragma unroll
         for (int v = 0; v < VPL; ++v) {
-          if (!on[v]) continue;
-          const uint32_t bits = word[v] >> sh[v];
-          acc[v].x += (bits & 1u) ? -cf : cf;
-          acc[v].y += (bits & 2u) ? -cf : cf;
-          acc[v].z += (bits & 4u) ? -cf : cf;
-          acc[v].w += (bits & 8u) ? -cf : cf;
+          const uint32_t bits = s_word[gi][k * 4 * NB + at[v]];
+          const uint32_t top = bits << sh[v];
+          acc[v].x += __uint_as_float(cf ^ ((top << 3) & 0x80000000u));
+          acc[v].y += __uint_as_float(cf ^ ((top << 2) & 0x80000000u));
+          acc[v].z += __uint_as_float(cf ^ ((top << 1) & 0x80000000u));
+          acc[v].w += __uint_as_float(cf ^ (top & 0x80000000u));
         }
       }
+      __syncwarp(gm);
     }
 #pragma unroll
     for (int v = 0; v < VPL; ++v) {
