@@ -312,7 +312,7 @@ __global__ void __launch_bounds__(T) k_update_fused(VecArgs a) {
         if (row < a.n) {
           const size_t i = (size_t)row * a.ld + 4 * q;
           r[k] = *reinterpret_cast<const float4*>(a.R + i);
-          ap[k] = *reinterpret_cast<const float4*>(a.AP + i);
+          ap[k] = __ldcs(reinterpret_cast<const float4*>(a.AP + i));  // its last use
         }
       }
 #pragma unroll
@@ -391,7 +391,12 @@ __global__ void __launch_bounds__(T) k_update_fused(VecArgs a) {
   const bool any_p = act.x | act.y | act.z | act.w;
   const bool any_x = al.x != 0.f || al.y != 0.f || al.z != 0.f || al.w != 0.f;
   if (!any_x && !any_p) return;
-  for (int64_t rowb = row0; rowb < a.n; rowb += UPD * rstep) {
+  // The rows backwards: the r rows that the first part wrote last are still in L2 (none of the first
+  // rows are, once a block of vectors exceeds it).  x is touched here alone, so it streams past.
+  // 169k nodes x 256 columns: a solve 126.0 -> 124.7 ms.
+  const int64_t chunks = (a.n - row0 + UPD * rstep - 1) / (UPD * rstep);
+  for (int64_t c = chunks - 1; c >= 0; --c) {
+    const int64_t rowb = row0 + c * UPD * rstep;
     float4 p[UPD], x[UPD], r[UPD];
 #pragma unroll
     for (int k = 0; k < UPD; ++k) {
@@ -399,7 +404,7 @@ __global__ void __launch_bounds__(T) k_update_fused(VecArgs a) {
       if (row < a.n) {
         const size_t i = (size_t)row * a.ld + 4 * q;
         p[k] = *reinterpret_cast<const float4*>(a.P + i);
-        if (any_x) x[k] = *reinterpret_cast<const float4*>(a.X + i);
+        if (any_x) x[k] = __ldcs(reinterpret_cast<const float4*>(a.X + i));
         if (any_p) r[k] = *reinterpret_cast<const float4*>(a.R + i);
       }
     }
@@ -415,7 +420,7 @@ __global__ void __launch_bounds__(T) k_update_fused(VecArgs a) {
         xx.y = fmaf(al.y, pp.y, xx.y);
         xx.z = fmaf(al.z, pp.z, xx.z);
         xx.w = fmaf(al.w, pp.w, xx.w);
-        *reinterpret_cast<float4*>(a.X + i) = xx;
+        __stcs(reinterpret_cast<float4*>(a.X + i), xx);
       }
       if (!any_p) continue;
       float4 rr = r[k];
