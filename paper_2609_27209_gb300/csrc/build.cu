@@ -144,7 +144,6 @@ __global__ void __launch_bounds__(BT)
     if (lane == 0) s_off[j][warp] = __popc(heads[j]);
   }
   __syncthreads();
-  volatile unsigned long long* st = status;
   if (warp == 0) {
     // 64 counts in key order (j, warp): two a lane
     static_assert(MERGE_IPT * (BT / 32) == 64, "two counts a lane");
@@ -159,35 +158,9 @@ __global__ void __launch_bounds__(BT)
     c[2 * lane] = inc - a - b;
     c[2 * lane + 1] = inc - b;
     const unsigned total = __shfl_sync(0xffffffffu, inc, 31);
+    const unsigned long long prefix = tile_prefix(status, t, total, spin_limit, abort);
     if (lane == 0) {
       s_total = total;
-      st[t] = (unsigned long long)total << 2 | (t == 0 ? 2ull : 1ull);
-    }
-    unsigned long long prefix = 0;
-    bool done = t == 0;
-    for (int64_t j = t - 1; !done; j -= 32) {
-      const int64_t q = j - lane;
-      unsigned long long x = 2ull;  // before tile 0: an inclusive prefix of 0
-      if (q >= 0) {
-        unsigned spins = 0;
-        while (((x = st[q]) & 3ull) == 0ull) {
-          if (++spins > spin_limit || aborted(abort)) {  // bounded: record it and take zero
-            atomicOr(abort, 1u);
-            x = 2ull;
-            break;
-          }
-        }
-      }
-      const unsigned incl = __ballot_sync(0xffffffffu, (x & 3ull) == 2ull);
-      const int stop = incl ? __ffs(incl) - 1 : 32;
-      unsigned long long part = lane <= stop ? x >> 2 : 0;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
-      prefix += part;
-      done = incl != 0;
-    }
-    if (lane == 0) {
-      if (t > 0) st[t] = (prefix + total) << 2 | 2ull;
       s_prefix = prefix;
     }
   }

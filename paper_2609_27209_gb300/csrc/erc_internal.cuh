@@ -259,6 +259,66 @@ __device__ __forceinline__ unsigned atom_add_acq_rel(unsigned* p, unsigned v) {
   return old;
 }
 
+// A call's abort word (device): a bounded wait that gives up sets it, and every later kernel of
+// the same call that would consume the unfinished result returns at once when it is set; the host
+// reads it once the call's work has finished and reports ERC_ERR_TIMEOUT.
+__device__ __forceinline__ bool aborted(const unsigned* abort) {
+  return *reinterpret_cast<const volatile unsigned*>(abort) != 0u;
+}
+
+// Decoupled look-back (D. Merrill, M. Garland, "Single-pass Parallel Prefix Scan with Decoupled
+// Look-back", 2016), called by one full warp of the block that holds tile t: publishes the tile's
+// `total` and returns the sum over the tiles before it.  Tiles are claimed in order through an
+// atomic ticket, so a tile only waits on tiles that have already started.  A status word is value
+// << 2 | flag (0 nothing yet, 1 the tile's total, 2 the sum up to and with it); the words are zero
+// at the start, the values non-negative and their sum below 2^62.  A trip reads the words of 128
+// tiles before: with 32 the walk back over the tiles in flight, one L2 latency a trip, bounded
+// the whole scan (64M flags: 0.9 ms).  Integer sums: the result does not depend on the order in
+// which tiles finish.
+// Every poll is bounded: after `spin_limit` polls (or once another tile has given up) the tile sets
+// the abort word and takes the predecessor as a final sum of zero, so its result stays within [0,
+// the true sum].
+__device__ __forceinline__ unsigned long long tile_prefix(volatile unsigned long long* st,
+                                                          int64_t t, unsigned long long total,
+                                                          unsigned spin_limit, unsigned* abort) {
+  constexpr int W = 4;
+  const int lane = threadIdx.x & 31;
+  if (lane == 0) st[t] = total << 2 | (t == 0 ? 2ull : 1ull);
+  if (t == 0) return 0;
+  unsigned long long prefix = 0;
+  for (int64_t j = t - 1;; j -= 32 * W) {
+    unsigned long long x[W];
+#pragma unroll
+    for (int i = 0; i < W; ++i) {
+      const int64_t q = j - 32 * i - lane;
+      x[i] = q >= 0 ? st[q] : 2ull;  // before tile 0: a final sum of 0
+    }
+#pragma unroll
+    for (int i = 0; i < W; ++i) {
+      const int64_t q = j - 32 * i - lane;
+      unsigned spins = 0;
+      while ((x[i] & 3ull) == 0ull) {
+        if (++spins > spin_limit || aborted(abort)) {
+          atomicOr(abort, 1u);
+          x[i] = 2ull;
+          break;
+        }
+        x[i] = st[q];
+      }
+      const unsigned incl = __ballot_sync(0xffffffffu, (x[i] & 3ull) == 2ull);
+      const int stop = incl ? __ffs(incl) - 1 : 32;  // the nearest final sum
+      unsigned long long part = lane <= stop ? x[i] >> 2 : 0;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+      prefix += part;
+      if (incl) {
+        if (lane == 0) st[t] = (prefix + total) << 2 | 2ull;
+        return prefix;
+      }
+    }
+  }
+}
+
 // Ordered column sums of G rows of partials (part: [G][ld] float pairs, written by other blocks
 // of the same launch, read through L2): threads take fixed segments of the rows for a pair of
 // columns each, every load of a chunk in flight, then the segments are added in order, so any
@@ -409,25 +469,11 @@ inline int grid_for(long long work_items, int items_per_block, int waves_blocks_
   return (int)g;
 }
 
-// A call's abort word (device): a bounded wait that gives up sets it, and every later kernel of
-// the same call that would consume the unfinished result returns at once when it is set; the host
-// reads it once the call's work has finished and reports ERC_ERR_TIMEOUT.
-__device__ __forceinline__ bool aborted(const unsigned* abort) {
-  return *reinterpret_cast<const volatile unsigned*>(abort) != 0u;
-}
-
 // ------------------------------------------------------------------------------------------------
 // internal entry points shared between translation units
 // ------------------------------------------------------------------------------------------------
 erc_status check_graph(const erc_graph* g);
 constexpr unsigned LOOKBACK_SPINS = 1u << 22;  // polls of a predecessor tile before giving up
-size_t scan_temp_bytes(int64_t n);
-// exclusive scan of int64 `in` (or of the 0/1 flags in `flags` when `in` is null) into `out`;
-// `total` (device, may be null) receives the sum.  `abort` (device, required) is the call's abort
-// word: the scan does nothing when it is already set, and sets it when a bounded look-back wait
-// gives up (the output is then incomplete; every entry stays within [0, the true value]).
-erc_status exclusive_scan_i64(const int64_t* in, const uint8_t* flags, int64_t* out, int64_t n,
-                              int64_t* total, void* tmp, cudaStream_t s, unsigned* abort);
 // Passes of a stable LSD radix sort of (key, value) pairs by 8-bit digits.  The caller zeroes the
 // temporary storage once (radix_sort_begin) and numbers its passes 0, 1, ..., also across several
 // sorts that share it; n_max bounds every one of them.  A pass sorts by key bits [shift, shift +
