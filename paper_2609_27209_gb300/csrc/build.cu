@@ -12,7 +12,9 @@
 // Sorting one key an edge (and then the edges by half a key) moves less than half the bytes of
 // sorting both directions by whole keys, and every edge id is known where its slot is written: no
 // search in the partner row.  What bounds each kernel is HBM, except where noted.  65.6M input
-// edges, 2.45M nodes: 10.6 ms, of 43.5 ms before (both directions sorted, binary searches).
+// edges, 2.45M nodes: 9.4 ms, of 43.5 ms before (both directions sorted, binary searches).
+#include <algorithm>
+
 #include "erc_internal.cuh"
 
 namespace erc {
@@ -37,6 +39,11 @@ struct BuildPlan {
 
 constexpr int MERGE_IPT = 8;
 constexpr int MERGE_TILE = BT * MERGE_IPT;
+
+inline int bit_length(uint32_t x) { return x ? 32 - __builtin_clz(x) : 0; }
+// sort passes over a whole key (two ids) and over one id
+inline int key_passes(int32_t n) { return (2 * bit_length((uint32_t)n) + RS_BITS - 1) / RS_BITS; }
+inline int id_passes(int32_t n) { return (bit_length((uint32_t)n) + RS_BITS - 1) / RS_BITS; }
 
 void plan_build(Arena& a, BuildPlan& p, int32_t n, int64_t m_in) {
   p.keys = a.take<uint64_t>(m_in);
@@ -126,75 +133,81 @@ __global__ void __launch_bounds__(BT)
   __shared__ unsigned long long s_prefix;
   unsigned* abort = err + 2;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (threadIdx.x == 0) s_tile = aborted(abort) ? 0xffffffffu : atomicAdd(err + 3, 1u);
   counts_clear(h);
-  if (s_tile == 0xffffffffu) return;
-  const int64_t t = s_tile, base = t * MERGE_TILE;
-  uint64_t k[MERGE_IPT], before[MERGE_IPT];
-  unsigned heads[MERGE_IPT];
+  for (;;) {
+    if (threadIdx.x == 0) s_tile = aborted(abort) ? 0xffffffffu : atomicAdd(err + 3, 1u);
+    __syncthreads();
+    const int64_t t = s_tile, base = t * MERGE_TILE;
+    if (s_tile == 0xffffffffu || base >= m_in) break;
+    uint64_t k[MERGE_IPT], before[MERGE_IPT];
+    unsigned heads[MERGE_IPT];
 #pragma unroll
-  for (int j = 0; j < MERGE_IPT; ++j) {
-    const int64_t i = base + j * BT + threadIdx.x;
-    k[j] = i < m_in ? keys[i] : sent;
-    before[j] = i > 0 && i < m_in ? keys[i - 1] : sent;  // no key before the first
-  }
-#pragma unroll
-  for (int j = 0; j < MERGE_IPT; ++j) {
-    heads[j] = __ballot_sync(0xffffffffu, k[j] != sent && k[j] != before[j]);
-    if (lane == 0) s_off[j][warp] = __popc(heads[j]);
-  }
-  __syncthreads();
-  if (warp == 0) {
-    // 64 counts in key order (j, warp): two a lane
-    static_assert(MERGE_IPT * (BT / 32) == 64, "two counts a lane");
-    unsigned* c = &s_off[0][0];
-    const unsigned a = c[2 * lane], b = c[2 * lane + 1];
-    unsigned inc = a + b;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned x = __shfl_up_sync(0xffffffffu, inc, o);
-      if (lane >= o) inc += x;
+    for (int j = 0; j < MERGE_IPT; ++j) {
+      const int64_t i = base + j * BT + threadIdx.x;
+      k[j] = i < m_in ? keys[i] : sent;
+      before[j] = i > 0 && i < m_in ? keys[i - 1] : sent;  // no key before the first
     }
-    c[2 * lane] = inc - a - b;
-    c[2 * lane + 1] = inc - b;
-    const unsigned total = __shfl_sync(0xffffffffu, inc, 31);
-    const unsigned long long prefix = tile_prefix(status, t, total, spin_limit, abort);
-    if (lane == 0) {
-      s_total = total;
-      s_prefix = prefix;
-    }
-  }
-  __syncthreads();
-  const uint64_t mask = (1ull << B) - 1ull;
-  bool other = false;
 #pragma unroll
-  for (int j = 0; j < MERGE_IPT; ++j) {
-    if (!((heads[j] >> lane) & 1u)) continue;
-    const int64_t i = base + j * BT + threadIdx.x;
-    const uint32_t e =
-        (uint32_t)s_prefix + s_off[j][warp] + __popc(heads[j] & ((1u << lane) - 1u));
-    double acc = 0.0;
-    for (int64_t d = i; d < m_in && (d == i || keys[d] == k[j]); ++d) {
-      acc += wbits ? (double)__uint_as_float(wbits[d]) : 1.0;
-      if (dup_first) break;
+    for (int j = 0; j < MERGE_IPT; ++j) {
+      heads[j] = __ballot_sync(0xffffffffu, k[j] != sent && k[j] != before[j]);
+      if (lane == 0) s_off[j][warp] = __popc(heads[j]);
     }
-    const int32_t u = (int32_t)(k[j] >> B), v = (int32_t)(k[j] & mask);
-    eu[e] = u;
-    ev[e] = v;
-    wout[e] = (float)acc;
-    if (ew) ew[e] = (float)acc;
-    other |= (float)acc != 1.f;
-    const uint64_t vk = ((uint64_t)v << B) | (uint64_t)u;
-    vkeys[e] = vk;
-    vvals[e] = e;
-    counts_add(h, vk, B, vpasses);
-    // rows up to u start here unless the key before lies in the same row
-    const int32_t pu = before[j] == sent ? -1 : (int32_t)(before[j] >> B);
-    for (int32_t r = pu + 1; r <= u; ++r) upper[r] = e;
+    __syncthreads();
+    if (warp == 0) {
+      // 64 counts in key order (j, warp): two a lane
+      static_assert(MERGE_IPT * (BT / 32) == 64, "two counts a lane");
+      unsigned* c = &s_off[0][0];
+      const unsigned a = c[2 * lane], b = c[2 * lane + 1];
+      unsigned inc = a + b;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned x = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += x;
+      }
+      c[2 * lane] = inc - a - b;
+      c[2 * lane + 1] = inc - b;
+      const unsigned total = __shfl_sync(0xffffffffu, inc, 31);
+      const unsigned long long prefix = tile_prefix(status, t, total, spin_limit, abort);
+      if (lane == 0) {
+        s_total = total;
+        s_prefix = prefix;
+      }
+    }
+    __syncthreads();
+    const uint64_t mask = (1ull << B) - 1ull;
+    bool other = false;
+#pragma unroll
+    for (int j = 0; j < MERGE_IPT; ++j) {
+      if (!((heads[j] >> lane) & 1u)) continue;
+      const int64_t i = base + j * BT + threadIdx.x;
+      const uint32_t e =
+          (uint32_t)s_prefix + s_off[j][warp] + __popc(heads[j] & ((1u << lane) - 1u));
+      float merged = wbits ? __uint_as_float(wbits[i]) : 1.f;
+      if (!dup_first && i + 1 < m_in && keys[i + 1] == k[j]) {  // float64 only where a run is
+        double acc = (double)merged;
+        for (int64_t d = i + 1; d < m_in && keys[d] == k[j]; ++d)
+          acc += wbits ? (double)__uint_as_float(wbits[d]) : 1.0;
+        merged = (float)acc;
+      }
+      const int32_t u = (int32_t)(k[j] >> B), v = (int32_t)(k[j] & mask);
+      eu[e] = u;
+      ev[e] = v;
+      wout[e] = merged;
+      if (ew) ew[e] = merged;
+      other |= merged != 1.f;
+      const uint64_t vk = ((uint64_t)v << B) | (uint64_t)u;
+      vkeys[e] = vk;
+      vvals[e] = e;
+      counts_add(h, vk, B, vpasses);
+      // rows up to u start here unless the key before lies in the same row
+      const int32_t pu = before[j] == sent ? -1 : (int32_t)(before[j] >> B);
+      for (int32_t r = pu + 1; r <= u; ++r) upper[r] = e;
+    }
+    if (!wbits && __any_sync(0xffffffffu, other) && lane == 0) atomicOr(err + 1, 1u);
+    if (base + MERGE_TILE >= m_in && threadIdx.x == 0) *m_out = (int64_t)(s_prefix + s_total);
+    __syncthreads();
   }
-  if (!wbits && __any_sync(0xffffffffu, other) && lane == 0) atomicOr(err + 1, 1u);
   counts_flush(h, counts, vpasses);
-  if (base + MERGE_TILE >= m_in && threadIdx.x == 0) *m_out = (int64_t)(s_prefix + s_total);
 }
 
 // U of the rows after the last edge's (every row when there is no edge)
@@ -250,9 +263,25 @@ __global__ void __launch_bounds__(BT)
     row_ptr[r] = m > 0 ? (int64_t)upper[r] + (int64_t)lower[r] : 0;
 }
 
-// float64 sum of a row's weights, rounded once.  Eight lanes a row; a warp's rows of more than 256
-// neighbours are taken by the whole warp, one after another, so that a hub does not hold up its
-// warp at eight lanes (one thread a row before: 5.4 ms on 2.45M nodes, bound by the largest row).
+// A running sum in three float32 words, each addition's error carried to the next word exactly: at
+// least 70 bits, where float64 has 53.  GB300 adds float64 at a sixty-fourth of the float32 rate, and
+// the conversions run there too; three words take 13 float32 operations an addend.
+struct Sum3 {
+  float a = 0.f, b = 0.f, c = 0.f;
+  __device__ __forceinline__ void add(float x) {
+    const float2 s = df_two_sum(a, x);
+    const float2 t = df_two_sum(b, s.y);
+    a = s.x;
+    b = t.x;
+    c = __fadd_rn(c, t.y);
+  }
+  __device__ __forceinline__ double value() const { return (double)a + ((double)b + (double)c); }
+};
+
+// A row's weights summed to at least float64's precision, rounded once.  Eight lanes a row; a warp's
+// rows of more than 256 neighbours are taken by the whole warp, one after another, so that a hub
+// does not hold up its warp at eight lanes.  2.45M nodes, 64.3M edges: 367 us; 862 us with float64
+// sums, 5.4 ms with one thread a row.
 constexpr int DL = 8;
 __global__ void __launch_bounds__(BT)
     k_degree(const int64_t* __restrict__ row_ptr, const float* __restrict__ val, int32_t n,
@@ -262,25 +291,26 @@ __global__ void __launch_bounds__(BT)
   const int64_t r = gtid() / DL;
   const int64_t j0 = r < n ? row_ptr[r] : 0, j1 = r < n ? row_ptr[r + 1] : 0;
   const bool is_long = j1 - j0 > 256;
-  double acc = 0.0;
+  Sum3 sum;
   if (!is_long)
-    for (int64_t j = j0 + gl; j < j1; j += DL) acc += (double)val[j];
+#pragma unroll 4
+    for (int64_t j = j0 + gl; j < j1; j += DL) sum.add(__ldg(val + j));
+  double acc = sum.value();
 #pragma unroll
   for (int o = DL / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   for (unsigned todo = __ballot_sync(0xffffffffu, is_long && gl == 0); todo; todo &= todo - 1) {
     const int owner = __ffs(todo) - 1;
     const int64_t a = __shfl_sync(0xffffffffu, j0, owner), b = __shfl_sync(0xffffffffu, j1, owner);
-    double sum = 0.0;
+    Sum3 part;
 #pragma unroll 4
-    for (int64_t j = a + lane; j < b; j += 32) sum += (double)val[j];
+    for (int64_t j = a + lane; j < b; j += 32) part.add(__ldg(val + j));
+    double all = part.value();
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-    if (lane == owner) acc = sum;
+    for (int o = 16; o > 0; o >>= 1) all += __shfl_xor_sync(0xffffffffu, all, o);
+    if (lane == owner) acc = all;
   }
   if (gl == 0 && r < n) deg[r] = (float)acc;
 }
-
-inline int bit_length(uint32_t x) { return x ? 32 - __builtin_clz(x) : 0; }
 
 }  // namespace
 }  // namespace erc
@@ -316,13 +346,12 @@ erc_status erc::build_laplacian_impl(int32_t n, const int32_t* src, const int32_
   Arena a(reinterpret_cast<void*>((reinterpret_cast<uintptr_t>(ws) + 255) & ~uintptr_t(255)));
   BuildPlan p;
   plan_build(a, p, n, m_in);
-  ERC_TRY(radix_sort_open());
 
   // the launch sequence is replayed from a cached CUDA graph: a dozen or so kernels whose launch
   // overhead would otherwise exceed the run time of the small ones
   const int B = bit_length((uint32_t)n);  // 2^B > n - 1: every id fits, and the sentinel sorts last
   const uint64_t sent = (2 * B >= 64) ? ~0ull : ((1ull << (2 * B)) - 1ull);
-  const int passes = (2 * B + RS_BITS - 1) / RS_BITS, vpasses = (B + RS_BITS - 1) / RS_BITS;
+  const int passes = key_passes(n), vpasses = id_passes(n);
   unsigned* abort = p.err + 2;
   float* cval = val ? val : p.val;
   auto enqueue = [&](cudaStream_t cs) -> erc_status {
@@ -348,7 +377,8 @@ erc_status erc::build_laplacian_impl(int32_t n, const int32_t* src, const int32_
         std::swap(va, vb);
       }
       unsigned long long* vcounts = p.counts + pass * RADIX;
-      k_merge<<<(unsigned)tiles, BT, 0, cs>>>(
+      // blocks that take tiles until none is left, so that their digit counts are flushed once
+      k_merge<<<(unsigned)std::min<int64_t>(tiles, 6 * sm_count()), BT, 0, cs>>>(
           ka, va, m_in, n, B, sent, dup_policy == ERC_DUP_FIRST, vpasses, eu, ev, ew, p.w, kb,
           vb ? vb : p.vals_alt, p.upper, vcounts, p.status, p.m, p.err, wait_limit(LOOKBACK_SPINS));
       count_launches(1);

@@ -476,16 +476,13 @@ erc_status check_graph(const erc_graph* g);
 constexpr unsigned LOOKBACK_SPINS = 1u << 22;  // polls of a predecessor tile before giving up
 // Passes of a stable LSD radix sort of (key, value) pairs by 8-bit digits.  The caller zeroes the
 // temporary storage once (radix_sort_begin) and numbers its passes 0, 1, ..., also across several
-// sorts that share it; n_max bounds every one of them.  A pass sorts by key bits [shift, shift +
+// sorts that share it; n_max (at most 2^30) bounds every one of them.  A pass sorts by key bits [shift, shift +
 // 8) the first min(n_max, *n) pairs (all n_max when n, a device pointer, is null); vals may be null.
-// counts[RS_RADIX] (device) holds how many of those keys have each digit.  radix_sort_open raises the
-// kernel's shared-memory limit on the current device: once before the passes are enqueued or
-// captured.  `abort` as for the scan: once it is set no further pass runs and the result is
-// undefined.
+// counts[RS_RADIX] (device) holds how many of those keys have each digit.   `abort`: the call's
+// abort word; once it is set no further pass runs and the result is undefined.
 constexpr int RS_BITS = 8;
 constexpr int RS_MAX_PASSES = 16;
 size_t radix_sort_temp_bytes(int64_t n_max);
-erc_status radix_sort_open();
 erc_status radix_sort_begin(int64_t n_max, void* tmp, cudaStream_t s);
 erc_status radix_sort_pass(const uint64_t* keys, const uint32_t* vals, uint64_t* keys_out,
                            uint32_t* vals_out, int64_t n_max, const int64_t* n, int shift, int pass,

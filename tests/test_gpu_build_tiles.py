@@ -32,3 +32,11 @@ def test_build_long_runs_and_hubs():
         for policy in (erc.ERC_DUP_SUM, erc.ERC_DUP_FIRST):
             g, ref = build_both(n, src, dst, weights, policy)
             assert_graph_equal(g, ref)
+
+
+@pytest.mark.parametrize("m", [(2 << 20) - 1, 2 << 20, 342 * 6144 + 1])
+def test_build_large_sort_tiles(m):
+    """Around the input size from which the sort takes its large tiles."""
+    _, src, dst, w = synth.random_multigraph(300000, m, seed=m, weighted=m % 2 == 0)
+    g, ref = build_both(300000, src, dst, w)
+    assert_graph_equal(g, ref)
