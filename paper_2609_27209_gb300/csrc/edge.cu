@@ -16,16 +16,24 @@ __device__ __forceinline__ float4 ld_f4(const float* p) {
   return __ldg(reinterpret_cast<const float4*>(p));
 }
 
-// One group of LPR lanes walks a segment of consecutive canonical edges, EB edges at a time with
-// every row load of the batch issued before the first use.  Edges are sorted by their smaller
-// endpoint, so the X_u loads of a batch mostly hit L1.  The group owns each R_e it touches, so
-// the accumulation needs no atomics; per edge the column order and the lane tree are fixed.
+// One group of LPR lanes walks a segment of consecutive canonical edges, EB of them a step: the
+// lanes load the step's endpoint ids together, then every row load of the step is issued before the
+// first use.  Edges are sorted by their smaller endpoint u, so a row X_u is loaded once per run of
+// equal u within a step.  The EB sums are reduced over the lanes together: halves of the group
+// exchange halves of the edges, so a step takes about EB + log2(LPR) shuffles instead of EB
+// log2(LPR); every sum still adds the same pairs (lane l to lane l ^ LPR/2, then LPR/4, ...), so
+// its bits do not change.  The group owns each R_e it touches: no atomics.
+// The rows X_v are random reads, bound by HBM where X exceeds L2 (7.4 TB/s for such reads).  Four
+// edges a step and four blocks an SM: 2.45M nodes, 64.3M edges, 128 columns, distances to
+// probabilities: 7.73 -> 6.81 ms (eight edges 7.46 with three blocks and 8.01 with four; five blocks
+// 7.96), with both rows loaded for every edge before.
 template <int LPR, int VPL>
-__global__ void __launch_bounds__(T)
+__global__ void __launch_bounds__(T, VPL == 1 ? 4 : VPL == 2 ? 3 : 2)
     k_edge_resistance(const int32_t* __restrict__ eu, const int32_t* __restrict__ ev, int64_t m,
                       const float* __restrict__ X, int32_t ld, int32_t kc, float* __restrict__ R) {
   constexpr int SEG = 32;
-  constexpr int EB = VPL >= 4 ? 1 : 4 / VPL;
+  constexpr int EB = VPL <= 4 ? 4 / VPL : 1;
+  static_assert(EB <= LPR && SEG % EB == 0, "a lane an edge");
   const int gl = threadIdx.x & (LPR - 1);
   const int gpb = T / LPR;
   const int nvec = ld >> 2;
@@ -35,40 +43,71 @@ __global__ void __launch_bounds__(T)
        sg += (int64_t)gridDim.x * gpb) {
     const int64_t e0 = sg * SEG, e1 = min(m, e0 + SEG);
     for (int64_t eb = e0; eb < e1; eb += EB) {
-      float4 xu[EB][VPL], xv[EB][VPL];
-      float rold[EB];
+      int32_t u[EB], v[EB];
+      // edges past the end repeat the last one: their sums are dropped
+      const int64_t e = min(eb + min(gl, EB - 1), e1 - 1);
+      const int32_t lu = __ldg(eu + e), lv = __ldg(ev + e);
 #pragma unroll
       for (int k = 0; k < EB; ++k) {
-        const bool ok = eb + k < e1;
-        const int32_t u = ok ? __ldg(eu + eb + k) : 0, v = ok ? __ldg(ev + eb + k) : 0;
+        u[k] = __shfl_sync(gm, lu, k, LPR);
+        v[k] = __shfl_sync(gm, lv, k, LPR);
+      }
+      const bool writes = gl < EB && eb + gl < e1;
+      const float rold = writes ? R[eb + gl] : 0.f;
+      float s[EB];
+      float4 xv[EB][VPL], xu[EB][VPL];
+#pragma unroll
+      for (int k = 0; k < EB; ++k)
 #pragma unroll
         for (int t = 0; t < VPL; ++t) {
           const int q = gl + LPR * t;
-          const bool on = ok && q < nvec;
-          xu[k][t] = on ? ld_f4(X + (size_t)u * ld + 4 * q) : make_float4(0.f, 0.f, 0.f, 0.f);
-          xv[k][t] = on ? ld_f4(X + (size_t)v * ld + 4 * q) : make_float4(0.f, 0.f, 0.f, 0.f);
+          xv[k][t] = q < nvec ? ld_f4(X + (size_t)v[k] * ld + 4 * q) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
-        rold[k] = ok && gl == 0 ? R[eb + k] : 0.f;
-      }
 #pragma unroll
-      for (int k = 0; k < EB; ++k) {
-        float s = 0.f;
+      for (int k = 0; k < EB; ++k)
 #pragma unroll
         for (int t = 0; t < VPL; ++t) {
+          const int q = gl + LPR * t;
+          xu[k][t] = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (q < nvec && (k == 0 || u[k] != u[k - 1])) xu[k][t] = ld_f4(X + (size_t)u[k] * ld + 4 * q);
+        }
+#pragma unroll
+      for (int k = 0; k < EB; ++k) {
+        s[k] = 0.f;
+#pragma unroll
+        for (int t = 0; t < VPL; ++t) {
+          if (k > 0 && u[k] == u[k - 1]) xu[k][t] = xu[k - 1][t];
           const int cb = 4 * (gl + LPR * t);
           const float dx = cb + 0 < kc ? xu[k][t].x - xv[k][t].x : 0.f;
           const float dy = cb + 1 < kc ? xu[k][t].y - xv[k][t].y : 0.f;
           const float dz = cb + 2 < kc ? xu[k][t].z - xv[k][t].z : 0.f;
           const float dw = cb + 3 < kc ? xu[k][t].w - xv[k][t].w : 0.f;
-          s = fmaf(dx, dx, s);
-          s = fmaf(dy, dy, s);
-          s = fmaf(dz, dz, s);
-          s = fmaf(dw, dw, s);
+          s[k] = fmaf(dx, dx, s[k]);
+          s[k] = fmaf(dy, dy, s[k]);
+          s[k] = fmaf(dz, dz, s[k]);
+          s[k] = fmaf(dw, dw, s[k]);
         }
-#pragma unroll
-        for (int off = LPR / 2; off > 0; off >>= 1) s += __shfl_xor_sync(gm, s, off, LPR);
-        if (gl == 0 && eb + k < e1) R[eb + k] = rold[k] + s;
       }
+      // sums over the lanes: while a lane holds more than one edge, the half of the group with bit
+      // `off` set keeps the upper half of them; edge k ends with the lanes from k LPR / EB up
+#pragma unroll
+      for (int off = LPR / 2, held = EB; off > 0; off >>= 1) {
+        if (held > 1) {
+          const int half = held / 2;
+          const bool up = (gl & off) != 0;
+#pragma unroll
+          for (int k = 0; k < EB / 2; ++k) {
+            if (k >= half) break;
+            const float give = up ? s[k] : s[k + half], keep = up ? s[k + half] : s[k];
+            s[k] = keep + __shfl_xor_sync(gm, give, off, LPR);
+          }
+          held = half;
+        } else {
+          s[0] += __shfl_xor_sync(gm, s[0], off, LPR);
+        }
+      }
+      const float sum = __shfl_sync(gm, s[0], (gl * (LPR / EB)) & (LPR - 1), LPR);
+      if (writes) R[eb + gl] = rold + sum;
     }
   }
 }
@@ -282,8 +321,15 @@ __global__ void k_normalize(const int64_t* __restrict__ row_ptr, const double* _
       pr = row_ptr[u + 1] > row_ptr[u] ? uni : 0.0;
     prob_node[u] = (float)pr;
   }
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += stride)
-    prob_edge[e] = (float)((double)edge_weight(kappa[e], kmax) * inv_e);
+  // weight times 1 / total, the reciprocal as a float pair: the exact product with its high part and
+  // the product with its low part, rounded once, like the float64 product that GB300 would run at
+  // a sixty-fourth of the float32 rate (64.3M edges: 171 us, 423 us with it)
+  const float2 inv = df_from_double(inv_e);
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += stride) {
+    const float w = edge_weight(kappa[e], kmax);
+    const float p = __fmul_rn(w, inv.x);
+    prob_edge[e] = __fadd_rn(p, __fmaf_rn(w, inv.y, __fmaf_rn(w, inv.x, -p)));
+  }
 }
 
 }  // namespace
