@@ -440,8 +440,8 @@ __global__ void __launch_bounds__(T) k_update_fused(VecArgs a) {
 // a thread-block cluster of CS blocks owns a group of 16 columns for every row and runs the whole
 // solve of its group; clusters never wait on one another.  Block k of a cluster owns the rows
 // [b_k, b_k+1) (equal shares of the neighbour lists, at most rbmax rows): their r and Ap live in
-// its shared memory, x and p in global memory (p is gathered by the cluster's other blocks, from
-// L2).  Four lanes take one light row, a float4 of the group's columns each, so a neighbour costs
+// its shared memory, and with PX x and a copy of p too; p is in global memory (it is gathered by the
+// cluster's other blocks, from L2), and so is x without PX.  Four lanes take one light row, a float4 of the group's columns each, so a neighbour costs
 // one 64-byte line; the next row's bounds and column indices are fetched while the current row's
 // neighbours are in flight.  Rows heavier than H are split over the whole block.  Per-column dot
 // products are combined in a fixed order: within a block by warp shuffles and shared memory,
@@ -619,7 +619,7 @@ __device__ __forceinline__ float4 eps_fma4(float e, float4 p, float4 acc) {
                      fmaf(e, p.w, acc.w));
 }
 
-template <bool WEIGHTED>
+template <bool WEIGHTED, bool PX>
 __global__ void __launch_bounds__(CT, 1) k_cg_cluster(ClusterArgs a) {
   extern __shared__ __align__(16) float4 csm[];
   __shared__ ClusterShared cl;
@@ -633,6 +633,8 @@ __global__ void __launch_bounds__(CT, 1) k_cg_cluster(ClusterArgs a) {
   const int rbmax = a.rbmax;
   float4* rs = csm;                 // [rbmax][CL] r of own rows
   float4* aps = csm + CL * rbmax;   // [rbmax][CL] Ap of own rows
+  float4* ps = aps + CL * rbmax;    // [rbmax][CL] p and x of own rows (PX)
+  float4* xs = ps + CL * rbmax;
 
   // ---- row split: S equal shares of the neighbour lists, each of at most rbmax rows
   const int64_t nnz = a.row_ptr[a.n];
@@ -717,9 +719,13 @@ __global__ void __launch_bounds__(CT, 1) k_cg_cluster(ClusterArgs a) {
       if (cb + 2 >= a.kc) y.z = 0.f;
       if (cb + 3 >= a.kc) y.w = 0.f;
       *reinterpret_cast<float4*>(a.P + o) = y;
-      *reinterpret_cast<float4*>(a.X + o) = f4_zero();
+      if (!PX) *reinterpret_cast<float4*>(a.X + o) = f4_zero();
     }
     rs[i * CL + gl] = y;
+    if (PX) {
+      ps[i * CL + gl] = y;
+      xs[i * CL + gl] = f4_zero();
+    }
     dot4(d, y, y);
   }
   cluster_colsum(d, cl, 0, S);  // its barrier also publishes p to the cluster
@@ -744,6 +750,12 @@ __global__ void __launch_bounds__(CT, 1) k_cg_cluster(ClusterArgs a) {
   }
   int any = __syncthreads_or(tid < CW && cl.active[tid]);
 
+  // p of own row i (this lane's columns)
+  auto own_p = [&](int i) {
+    if (PX) return ps[i * CL + gl];
+    return valid ? __ldcg(reinterpret_cast<const float4*>(a.P + (size_t)(b0 + i) * a.ld + qoff))
+                 : f4_zero();
+  };
   int slot = 1;
   while (any) {
     // ---------------- A: Ap = L_eps p on own rows, p.Ap
@@ -775,9 +787,7 @@ __global__ void __launch_bounds__(CT, 1) k_cg_cluster(ClusterArgs a) {
           nnj1 = rp[i + 2 * CGR + 1];
         }
         if (!hv) {
-          const float4 pu = valid ? __ldcg(reinterpret_cast<const float4*>(
-                                        a.P + (size_t)(b0 + i) * a.ld + qoff))
-                                  : f4_zero();
+          const float4 pu = own_p(i);
           float4 acc = f4_zero();
           cluster_batch<WEIGHTED>(a, valid, qoff, pu, c, w, j0, j1, gm, acc);
           for (int64_t jb = j0 + CU; jb < j1; jb += CU) {  // rows longer than one batch
@@ -805,9 +815,7 @@ __global__ void __launch_bounds__(CT, 1) k_cg_cluster(ClusterArgs a) {
       const int64_t j0 = rp[i], j1 = rp[i + 1];
       const int64_t per = (j1 - j0 + CGR - 1) / CGR;
       const int64_t s0 = min(j1, j0 + gi * per), s1 = min(j1, s0 + per);
-      const float4 pu = valid ? __ldcg(reinterpret_cast<const float4*>(
-                                    a.P + (size_t)(b0 + i) * a.ld + qoff))
-                              : f4_zero();
+      const float4 pu = own_p(i);
       float4 acc = f4_zero();
       int c[CIDX];
       float w[CIDX];
@@ -868,17 +876,20 @@ __global__ void __launch_bounds__(CT, 1) k_cg_cluster(ClusterArgs a) {
           for (int k = 0; k < CUNROLL; ++k) {
             const int i = i0 + k * CGR;
             if (i < nr) {
-              const size_t o = (size_t)(b0 + i) * a.ld + qoff;
-              p[k] = __ldcg(reinterpret_cast<const float4*>(a.P + o));
-              x[k] = *reinterpret_cast<const float4*>(a.X + o);
+              p[k] = own_p(i);
+              x[k] = PX ? xs[i * CL + gl]
+                        : *reinterpret_cast<const float4*>(a.X + (size_t)(b0 + i) * a.ld + qoff);
             }
           }
 #pragma unroll
           for (int k = 0; k < CUNROLL; ++k) {
             const int i = i0 + k * CGR;
             if (i < nr) {
-              const size_t o = (size_t)(b0 + i) * a.ld + qoff;
-              *reinterpret_cast<float4*>(a.X + o) = fma4(al, p[k], x[k]);
+              const float4 xn = fma4(al, p[k], x[k]);
+              if (PX)
+                xs[i * CL + gl] = xn;
+              else
+                *reinterpret_cast<float4*>(a.X + (size_t)(b0 + i) * a.ld + qoff) = xn;
               const float4 r = fma4(nal, aps[i * CL + gl], rs[i * CL + gl]);
               rs[i * CL + gl] = r;
               dot4(d, r, r);
@@ -928,8 +939,7 @@ __global__ void __launch_bounds__(CT, 1) k_cg_cluster(ClusterArgs a) {
 #pragma unroll
           for (int k = 0; k < CUNROLL; ++k) {
             const int i = i0 + k * CGR;
-            if (i < nr)
-              p[k] = __ldcg(reinterpret_cast<const float4*>(a.P + (size_t)(b0 + i) * a.ld + qoff));
+            if (i < nr) p[k] = own_p(i);
           }
 #pragma unroll
           for (int k = 0; k < CUNROLL; ++k) {
@@ -941,6 +951,7 @@ __global__ void __launch_bounds__(CT, 1) k_cg_cluster(ClusterArgs a) {
               if (act.z) p[k].z = fmaf(be.z, p[k].z, r.z);
               if (act.w) p[k].w = fmaf(be.w, p[k].w, r.w);
               *reinterpret_cast<float4*>(a.P + (size_t)(b0 + i) * a.ld + qoff) = p[k];
+              if (PX) ps[i * CL + gl] = p[k];
             }
           }
         }
@@ -948,6 +959,9 @@ __global__ void __launch_bounds__(CT, 1) k_cg_cluster(ClusterArgs a) {
     }
     cluster_barrier();
   }
+  if (PX && valid)
+    for (int i = gi; i < nr; i += CGR)
+      *reinterpret_cast<float4*>(a.X + (size_t)(b0 + i) * a.ld + qoff) = xs[i * CL + gl];
   // no block leaves while another may still read its partials
   cluster_barrier();
   const int c = 4 * CL * (int)cluster_index() + tid;
@@ -1213,15 +1227,19 @@ void cluster_config(const ClusterPlan& pl, cudaStream_t s, cudaLaunchConfig_t* c
   cfg->numAttrs = 1;
 }
 
-bool cluster_plan(const erc_graph* g, int ld, ClusterPlan* pl) {
-  const void* k = g->val ? (const void*)k_cg_cluster<true> : (const void*)k_cg_cluster<false>;
+bool cluster_plan_for(const erc_graph* g, int ld, bool px, ClusterPlan* pl) {
+  const void* k = g->val ? (px ? (const void*)k_cg_cluster<true, true>
+                               : (const void*)k_cg_cluster<true, false>)
+                         : (px ? (const void*)k_cg_cluster<false, true>
+                               : (const void*)k_cg_cluster<false, false>);
   const size_t lim = open_smem(k);
   if (!lim || cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
                   cudaSuccess) {
     cudaGetLastError();
     return false;
   }
-  const int64_t row_bytes = 2 * CL * sizeof(float4);  // r and Ap of the group's columns
+  // r and Ap (and p and x) of the group's columns
+  const int64_t row_bytes = (px ? 4 : 2) * CL * sizeof(float4);
   const int64_t cap = ((int64_t)lim - 1024) / row_bytes;
   const int groups = (ld / 4 + CL - 1) / CL;
   for (int S = CMAXS; S >= 1; --S) {
@@ -1246,6 +1264,16 @@ bool cluster_plan(const erc_graph* g, int ld, ClusterPlan* pl) {
     return true;
   }
   return false;
+}
+
+// The largest cluster decides (it is what the solve's time depends on); where the same one and the
+// same row split hold p and x of a block's rows in shared memory too, they stay there: the vector phases then wait on no load
+// (2,000 nodes, 64 columns: 282 us a solve, 300 us with both in L2).
+bool cluster_plan(const erc_graph* g, int ld, ClusterPlan* pl) {
+  ClusterPlan px;
+  if (!cluster_plan_for(g, ld, false, pl)) return false;
+  if (cluster_plan_for(g, ld, true, &px) && px.S == pl->S && px.rbmax == pl->rbmax) *pl = px;
+  return true;
 }
 
 // Both single-launch plans for a graph shape, computed once per (device, n, ld, weighted,
