@@ -1432,12 +1432,10 @@ erc_status iteration_graph(const SpmmArgs& sa, int sgrid, const VecArgs& va, int
   return ERC_OK;
 }
 
-int iterations_per_poll(const erc_graph* g, int ld) {
-  const double bytes = (double)(2 * g->m + g->n) * ld * 4.0;  // gathered + streamed per iteration
-  if (bytes < 256e6) return 16;
-  if (bytes < 2e9) return 4;
-  return 2;
-}
+// Iterations between two looks at the "any column active" flag.  A look costs the stream about 15
+// us of idling (the copy, the host's wake-up, the next launch); an iteration past the end costs two
+// kernels that return at once, about 6 us.
+constexpr int ITERS_PER_POLL = 8;
 
 erc_status check_block(const float* p, const char* name) {
   ERC_REQUIRE(p && (reinterpret_cast<uintptr_t>(p) & 15) == 0, "%s must be 16-byte aligned", name);
@@ -1588,7 +1586,7 @@ erc_status erc::cg_enqueue(const erc_graph* g, float eps, const float* Y, float*
     ra.v.spin_limit = wait_limit(RES_SPIN_LIMIT);
     ERC_TRY(launch_resident(kres, ra, smem, s));
   } else {
-    const int S = iterations_per_poll(g, ld);
+    const int S = ITERS_PER_POLL;
     cudaGraphExec_t exec = nullptr;
     ERC_TRY(iteration_graph(sa, sgrid, va, ugrid, S, &exec));
     int done = 0;
