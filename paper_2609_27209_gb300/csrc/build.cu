@@ -12,7 +12,7 @@
 // Sorting one key an edge (and then the edges by half a key) moves less than half the bytes of
 // sorting both directions by whole keys, and every edge id is known where its slot is written: no
 // search in the partner row.  What bounds each kernel is HBM, except where noted.  65.6M input
-// edges, 2.45M nodes: 9.4 ms, of 43.5 ms before (both directions sorted, binary searches).
+// edges, 2.45M nodes: 9.1 ms, of 43.5 ms before (both directions sorted, binary searches).
 #include <algorithm>
 
 #include "erc_internal.cuh"
@@ -38,6 +38,7 @@ struct BuildPlan {
 };
 
 constexpr int MERGE_IPT = 8;
+constexpr int MERGE_BLOCKS = 4;  // per SM
 constexpr int MERGE_TILE = BT * MERGE_IPT;
 
 inline int bit_length(uint32_t x) { return x ? 32 - __builtin_clz(x) : 0; }
@@ -119,7 +120,7 @@ __global__ void __launch_bounds__(BT)
 // counts (as in the scan; a word is count << 2 | flag).  The head's thread merges its run: the
 // float64 sum of the duplicates' weights in input order (the sort is stable), rounded once.  Also
 // written: U, the edges as keys (v << B | u) for the sort by v, and that sort's digit counts.
-__global__ void __launch_bounds__(BT)
+__global__ void __launch_bounds__(BT, MERGE_BLOCKS)
     k_merge(const uint64_t* __restrict__ keys, const uint32_t* __restrict__ wbits, int64_t m_in,
             int32_t n, int B, uint64_t sent, int dup_first, int vpasses, int32_t* __restrict__ eu,
             int32_t* __restrict__ ev, float* __restrict__ ew, float* __restrict__ wout,
@@ -378,7 +379,7 @@ erc_status erc::build_laplacian_impl(int32_t n, const int32_t* src, const int32_
       }
       unsigned long long* vcounts = p.counts + pass * RADIX;
       // blocks that take tiles until none is left, so that their digit counts are flushed once
-      k_merge<<<(unsigned)std::min<int64_t>(tiles, 6 * sm_count()), BT, 0, cs>>>(
+      k_merge<<<(unsigned)std::min<int64_t>(tiles, MERGE_BLOCKS * sm_count()), BT, 0, cs>>>(
           ka, va, m_in, n, B, sent, dup_policy == ERC_DUP_FIRST, vpasses, eu, ev, ew, p.w, kb,
           vb ? vb : p.vals_alt, p.upper, vcounts, p.status, p.m, p.err, wait_limit(LOOKBACK_SPINS));
       count_launches(1);
