@@ -12,7 +12,7 @@
 // A subgraph is drawn for every training step, so passes and round trips count: the weights are
 // formed inside the scan, a draw marks at once, and a compaction is one pass that reads the marks
 // (or tests the endpoints), finds its place by look-back and writes the ids.  169k nodes, 16,934
-// draws and the subgraph's counts: 182 us, 233 us before; 64.3M edges, 6.4M draws: 2.24 ms, 3.96 ms
+// draws and the subgraph's counts: 164 us, 232 us before; 64.3M edges, 6.4M draws: 1.44 ms, 3.95 ms
 // before, with separate passes for weights, draws, marks, induced flags, scans and compactions and
 // two round trips.
 #include "erc_internal.cuh"
@@ -22,22 +22,35 @@ namespace {
 
 constexpr int ST = 256;
 constexpr int SWARPS = ST / 32;
-constexpr int SIPT = 32;               // entries per thread of a scan or compaction tile: few tiles, so
-constexpr int STILE = ST * SIPT;       // that the look-back over those in flight stays short
+// Entries per thread of a scan or compaction tile: 32 from SLARGE entries on, so that the look-back
+// over the tiles in flight stays short, 8 below, so that a small graph's passes spread over the SMs.
+constexpr int SIPT_LARGE = 32, SIPT_SMALL = 8;
+constexpr int64_t SLARGE = 1 << 20;
+constexpr int SMID = 64;
 constexpr uint32_t SAMPLER_TAG = 0x53414D50u;
 
 struct SamplePlan {
-  int64_t *E, *totals;  // totals: [0] T [1] nodes [2] edges
+  int64_t *E, *Emid, *totals;  // Emid: every SMID-th entry of E; totals: [0] T [1] nodes [2] edges
   uint8_t *nmark, *emark;
+  uint32_t* nbits;             // the node marks as bits
   unsigned long long* status;  // look-back words of the three passes
   unsigned* err;  // [0] a probability outside [0, 1]; [1] the abort word; [2..4] the passes' tickets
 };
 
-inline int64_t stiles(int64_t count) { return (count + STILE - 1) / STILE; }
+inline int64_t stile(int64_t count) { return ST * (count < SLARGE ? SIPT_SMALL : SIPT_LARGE); }
+inline int64_t stiles(int64_t count) { return (count + stile(count) - 1) / stile(count); }
+
+// copies of the node marks: at most 16, and 64 MB of them
+inline int mark_copies(int32_t n) {
+  const int64_t c = (int64_t(64) << 20) / n;
+  return c < 1 ? 1 : c > 16 ? 16 : (int)c;
+}
 
 void plan_sample(Arena& a, SamplePlan& p, int64_t count, int32_t n, int64_t m) {
   p.E = a.take<int64_t>(count);
-  p.nmark = a.take<uint8_t>(n);
+  p.Emid = a.take<int64_t>(count / SMID + 1);
+  p.nmark = a.take<uint8_t>((size_t)n * mark_copies(n));
+  p.nbits = a.take<uint32_t>((size_t)n / 32 + 1);
   p.emark = a.take<uint8_t>(m > 0 ? m : 1);
   p.totals = a.take<int64_t>(4);
   p.err = a.take<unsigned>(8);
@@ -67,23 +80,39 @@ __device__ __forceinline__ int64_t claim_tile(unsigned* ticket, const unsigned* 
   return s_tile == 0xffffffffu ? -1 : (int64_t)s_tile;
 }
 
-// E and T of the weights.  A warp takes 32 SIPT consecutive entries, 32 at a time.
+// E, Emid and T of the weights.  A warp takes 32 SIPT consecutive entries, a lane four neighbouring
+// ones of each 128, so that a scan over the lanes serves 128 entries; `vec`: prob is 16-byte aligned.
+template <int SIPT>
 __global__ void __launch_bounds__(ST)
-    k_weight_scan(const float* __restrict__ prob, int64_t count, int64_t* __restrict__ E,
-                  int64_t* __restrict__ total, unsigned long long* status, unsigned* err,
-                  unsigned spin_limit) {
+    k_weight_scan(const float* __restrict__ prob, int64_t count, bool vec, int64_t* __restrict__ E,
+                  int64_t* __restrict__ Emid, int64_t* __restrict__ total,
+                  unsigned long long* status, unsigned* err, unsigned spin_limit) {
+  constexpr int64_t STILE = ST * SIPT;
   __shared__ unsigned long long s_warp[SWARPS], s_prefix, s_total;
   const int64_t t = claim_tile(err + 2, err + 1);
   if (t < 0) return;
+  constexpr int ROUNDS = SIPT / 4;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t base = t * STILE + (int64_t)warp * 32 * SIPT + lane;
-  float p[SIPT];
+  const int64_t base = t * STILE + (int64_t)warp * 32 * SIPT + 4 * lane;
+  float4 p[ROUNDS];
 #pragma unroll
-  for (int j = 0; j < SIPT; ++j) p[j] = base + 32 * j < count ? prob[base + 32 * j] : 0.f;
+  for (int j = 0; j < ROUNDS; ++j) {
+    const int64_t i = base + 128 * j;
+    if (vec && i + 4 <= count) {
+      p[j] = __ldg(reinterpret_cast<const float4*>(prob + i));
+    } else {
+      p[j].x = i + 0 < count ? prob[i + 0] : 0.f;
+      p[j].y = i + 1 < count ? prob[i + 1] : 0.f;
+      p[j].z = i + 2 < count ? prob[i + 2] : 0.f;
+      p[j].w = i + 3 < count ? prob[i + 3] : 0.f;
+    }
+  }
   bool bad = false;
   unsigned long long sum = 0;
 #pragma unroll
-  for (int j = 0; j < SIPT; ++j) sum += fixed_weight(p[j], bad);
+  for (int j = 0; j < ROUNDS; ++j)
+    sum += fixed_weight(p[j].x, bad) + fixed_weight(p[j].y, bad) + fixed_weight(p[j].z, bad) +
+           fixed_weight(p[j].w, bad);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
   if (lane == 0) s_warp[warp] = sum;
@@ -107,30 +136,51 @@ __global__ void __launch_bounds__(ST)
   __syncthreads();
   unsigned long long run = s_prefix + s_warp[warp];
 #pragma unroll
-  for (int j = 0; j < SIPT; ++j) {
-    const unsigned long long w = fixed_weight(p[j], bad);
+  for (int j = 0; j < ROUNDS; ++j) {
+    const int64_t i = base + 128 * j;
+    const unsigned long long w0 = fixed_weight(p[j].x, bad), w1 = fixed_weight(p[j].y, bad),
+                             w2 = fixed_weight(p[j].z, bad), w3 = fixed_weight(p[j].w, bad);
+    const unsigned long long w = w0 + w1 + w2 + w3;
     unsigned long long inc = w;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const unsigned long long x = __shfl_up_sync(0xffffffffu, inc, o);
       if (lane >= o) inc += x;
     }
-    if (base + 32 * j < count) E[base + 32 * j] = (int64_t)(run + inc - w);
+    const unsigned long long e0 = run + inc - w, e1 = e0 + w0, e2 = e1 + w1, e3 = e2 + w2;
+    if (i + 4 <= count) {
+      *reinterpret_cast<ulonglong2*>(E + i) = make_ulonglong2(e0, e1);
+      *reinterpret_cast<ulonglong2*>(E + i + 2) = make_ulonglong2(e2, e3);
+    } else {
+      if (i + 0 < count) E[i + 0] = (int64_t)e0;
+      if (i + 1 < count) E[i + 1] = (int64_t)e1;
+      if (i + 2 < count) E[i + 2] = (int64_t)e2;
+    }
+    if (lane % (SMID / 4) == 0 && i < count) Emid[i / SMID] = (int64_t)e0;
     run += __shfl_sync(0xffffffffu, inc, 31);
   }
   if ((t + 1) * STILE >= count && threadIdx.x == 0) *total = (int64_t)s_total;
 }
 
-// draw k: the largest i with E_i <= floor(x_k T / 2^64); marks node i, or edge i's endpoints and,
-// where emark is not null, the edge.  A mark is tested first: most draws of a power-law graph's
-// endpoints find theirs set, and a cached read is cheaper than a byte store.
+// draw k: the largest i with E_i <= floor(x_k T / 2^64), found in the scan's tiles (their final status
+// words hold the sums with each tile: a few KB that stay in L1), then in Emid (L2), then among the
+// SMID entries of E it leads to: a plain binary search over E misses L2 about eight times a draw
+// on 64M entries.  Marks node i, or edge i's endpoints and, where emark is not null, the edge.
+// Stores to one line queue up in L2, and a power-law graph's draws keep hitting the lines of its
+// hubs: the blocks spread them over `copies` arrays of marks, which the compaction joins.  (Testing a
+// mark before storing it queues the test behind the stores: 276 us against 31 for 129k draws
+// over 6,821 nodes.)
 __global__ void __launch_bounds__(ST)
-    k_draw(const int64_t* __restrict__ E, int64_t count, const int64_t* __restrict__ tot,
+    k_draw(const int64_t* __restrict__ E, const int64_t* __restrict__ Emid, int64_t count, int64_t tile,
+           const unsigned long long* __restrict__ status, const int64_t* __restrict__ tot,
            int64_t budget, uint2 key, int64_t first, uint32_t stream,
-           const int32_t* __restrict__ eu, const int32_t* __restrict__ ev, uint8_t* nmark,
-           uint8_t* emark, const unsigned* abort) {
+           const int32_t* __restrict__ eu, const int32_t* __restrict__ ev,
+           uint8_t* __restrict__ nmark, int32_t n, int copies, uint8_t* __restrict__ emark,
+           const unsigned* abort) {
   if (aborted(abort)) return;
+  nmark += (size_t)(blockIdx.x % copies) * n;
   const uint64_t T = (uint64_t)tot[0];
+  const int64_t tiles = (count + tile - 1) / tile;
   for (int64_t k = (int64_t)blockIdx.x * ST + threadIdx.x; k < budget;
        k += (int64_t)gridDim.x * ST) {
     const uint64_t d = (uint64_t)(first + k);
@@ -138,19 +188,33 @@ __global__ void __launch_bounds__(ST)
         philox4x32_10(make_uint4((uint32_t)d, (uint32_t)(d >> 32), SAMPLER_TAG, stream), key);
     const uint64_t x = ((uint64_t)w.x << 32) | w.y;
     const int64_t r = (int64_t)__umul64hi(x, T);
-    int64_t lo = 0, hi = count;  // first index with E > r, minus one
+    int64_t lo = 0, hi = tiles - 1;  // first tile whose sum with it exceeds r
     while (lo < hi) {
       const int64_t mid = (lo + hi) >> 1;
-      if (E[mid] <= r) lo = mid + 1; else hi = mid;
+      if ((int64_t)(__ldg(status + mid) >> 2) > r) hi = mid; else lo = mid + 1;
     }
-    const int64_t i = lo - 1;
+    // the last of Emid, then of E, with E <= r (the first of each range always is)
+    const int64_t tile_end = min(count, (lo + 1) * tile);
+    lo = lo * (tile / SMID);
+    hi = (tile_end - 1) / SMID;
+    while (lo < hi) {
+      const int64_t mid = (lo + hi + 1) >> 1;
+      if (Emid[mid] <= r) lo = mid; else hi = mid - 1;
+    }
+    lo = lo * SMID;
+    hi = min(tile_end, lo + SMID) - 1;
+    while (lo < hi) {
+      const int64_t mid = (lo + hi + 1) >> 1;
+      if (E[mid] <= r) lo = mid; else hi = mid - 1;
+    }
+    const int64_t i = lo;
     if (stream) {
       if (emark) emark[i] = 1;
       const int32_t u = eu[i], v = ev[i];
-      if (!__ldcg(nmark + u)) nmark[u] = 1;
-      if (!__ldcg(nmark + v)) nmark[v] = 1;
+      nmark[u] = 1;
+      nmark[v] = 1;
     } else {
-      if (!__ldcg(nmark + i)) nmark[i] = 1;
+      nmark[i] = 1;
     }
   }
 }
@@ -159,19 +223,33 @@ struct MarkedFlag {
   const uint8_t* mark;
   __device__ bool operator()(int64_t i) const { return mark[i] != 0; }
 };
+struct CopiesFlag {  // marked in any of the copies, `n` apart
+  const uint8_t* mark;
+  int64_t n;
+  int copies;
+  __device__ bool operator()(int64_t i) const {
+    unsigned any = 0;
+    for (int c = 0; c < copies; ++c) any |= mark[c * n + i];
+    return any != 0;
+  }
+};
 struct InducedFlag {  // both endpoints of edge i are marked
   const int32_t *eu, *ev;
-  const uint8_t* nmark;
+  const uint32_t* nbits;
   __device__ bool operator()(int64_t i) const {
-    return __ldg(nmark + eu[i]) & __ldg(nmark + ev[i]);
+    const int32_t u = __ldg(eu + i), v = __ldg(ev + i);
+    return (__ldg(nbits + (u >> 5)) >> (u & 31)) & (__ldg(nbits + (v >> 5)) >> (v & 31)) & 1u;
   }
 };
 
-// the ids i < count with flag(i), ascending
-template <class Flag>
+// the ids i < count with flag(i), ascending, and the flags as bits where `bits` is not null (an
+// eighth of the marks' bytes: 2.4M nodes' bits mostly stay in L1 while the edges test them)
+template <int SIPT, class Flag>
 __global__ void __launch_bounds__(ST)
-    k_compact(Flag flag, int64_t count, int32_t* __restrict__ out, int64_t* __restrict__ total,
+    k_compact(Flag flag, int64_t count, int32_t* __restrict__ out, uint32_t* __restrict__ bits,
+              int64_t* __restrict__ total,
               unsigned long long* status, unsigned* ticket, unsigned* abort, unsigned spin_limit) {
+  constexpr int64_t STILE = ST * SIPT;
   __shared__ unsigned s_warp[SWARPS];
   __shared__ unsigned long long s_prefix, s_total;
   const int64_t t = claim_tile(ticket, abort);
@@ -187,7 +265,8 @@ __global__ void __launch_bounds__(ST)
     if (lane == j) mine = bal;
     cnt += __popc(bal);
   }
-  static_assert(SIPT == 32, "a lane holds one ballot");
+  if (bits && lane < SIPT && base + 32 * lane < count) bits[(base >> 5) + lane] = mine;
+  static_assert(SIPT <= 32, "a lane holds one ballot");
   if (lane == 0) s_warp[warp] = cnt;
   __syncthreads();
   if (warp == 0) {
@@ -244,6 +323,22 @@ __global__ void k_saint_norm(const int64_t* __restrict__ row_ptr,
   }
 }
 
+template <class Flag>
+erc_status compact(Flag flag, int64_t count, int32_t* out, uint32_t* bits, int64_t* total,
+                   unsigned long long* status, unsigned* ticket, unsigned* abort, unsigned limit,
+                   cudaStream_t s) {
+  const unsigned grid = (unsigned)stiles(count);
+  if (count < SLARGE)
+    k_compact<SIPT_SMALL><<<grid, ST, 0, s>>>(flag, count, out, bits, total, status, ticket, abort,
+                                              limit);
+  else
+    k_compact<SIPT_LARGE><<<grid, ST, 0, s>>>(flag, count, out, bits, total, status, ticket, abort,
+                                              limit);
+  count_launches(1);
+  ERC_CUDA(cudaGetLastError());
+  return ERC_OK;
+}
+
 }  // namespace
 }  // namespace erc
 
@@ -289,36 +384,37 @@ extern "C" erc_status erc_sample_subgraph(const erc_graph* g, int32_t kind, cons
   ERC_CUDA(cudaMemsetAsync(p.status, 0,
                            (size_t)(stiles(count) + stiles(g->n) + stiles(g->m)) *
                                sizeof(unsigned long long), s));
-  ERC_CUDA(cudaMemsetAsync(p.nmark, 0, (size_t)g->n, s));
+  const int copies = mark_copies(g->n);
+  ERC_CUDA(cudaMemsetAsync(p.nmark, 0, (size_t)g->n * copies, s));
   if (drawn_edges) ERC_CUDA(cudaMemsetAsync(p.emark, 0, (size_t)g->m, s));
   // Nothing is read back before the end: a probability outside [0, 1] counts as zero, with a total of
   // zero every draw is the last index, and the prefixes are only ever below their true values when
   // a bounded wait gives up, so every index stays in range; the host then reports the error.
   const unsigned limit = wait_limit(LOOKBACK_SPINS);
-  k_weight_scan<<<(unsigned)stiles(count), ST, 0, s>>>(prob, count, p.E, &p.totals[0], p.status,
-                                                       p.err, limit);
+  const bool vec = (reinterpret_cast<uintptr_t>(prob) & 15) == 0;
+  if (count < SLARGE)
+    k_weight_scan<SIPT_SMALL><<<(unsigned)stiles(count), ST, 0, s>>>(
+        prob, count, vec, p.E, p.Emid, &p.totals[0], p.status, p.err, limit);
+  else
+    k_weight_scan<SIPT_LARGE><<<(unsigned)stiles(count), ST, 0, s>>>(
+        prob, count, vec, p.E, p.Emid, &p.totals[0], p.status, p.err, limit);
   count_launches(1);
   ERC_CUDA(cudaGetLastError());
   const uint2 key = make_uint2((uint32_t)(seed & 0xffffffffu), (uint32_t)(seed >> 32));
-  k_draw<<<grid_for(budget, ST), ST, 0, s>>>(p.E, count, p.totals, budget, key, first_draw,
-                                             by_edge ? 1u : 0u, g->eu, g->ev, p.nmark,
-                                             drawn_edges ? p.emark : nullptr, abort);
+  k_draw<<<grid_for(budget, ST), ST, 0, s>>>(p.E, p.Emid, count, stile(count), p.status, p.totals, budget, key, first_draw,
+                                             by_edge ? 1u : 0u, g->eu, g->ev, p.nmark, g->n,
+                                             copies, drawn_edges ? p.emark : nullptr, abort);
   count_launches(1);
   ERC_CUDA(cudaGetLastError());
-  k_compact<<<(unsigned)stiles(g->n), ST, 0, s>>>(MarkedFlag{p.nmark}, (int64_t)g->n, nodes,
-                                                  &p.totals[1], st_n, p.err + 3, abort, limit);
-  count_launches(1);
-  ERC_CUDA(cudaGetLastError());
+  ERC_TRY(compact(CopiesFlag{p.nmark, g->n, copies}, (int64_t)g->n, nodes, p.nbits, &p.totals[1],
+                  st_n, p.err + 3, abort, limit, s));
   if (g->m > 0) {
     if (drawn_edges)
-      k_compact<<<(unsigned)stiles(g->m), ST, 0, s>>>(MarkedFlag{p.emark}, g->m, edges,
-                                                      &p.totals[2], st_m, p.err + 4, abort, limit);
+      ERC_TRY(compact(MarkedFlag{p.emark}, g->m, edges, (uint32_t*)nullptr, &p.totals[2], st_m,
+                      p.err + 4, abort, limit, s));
     else
-      k_compact<<<(unsigned)stiles(g->m), ST, 0, s>>>(InducedFlag{g->eu, g->ev, p.nmark}, g->m,
-                                                      edges, &p.totals[2], st_m, p.err + 4, abort,
-                                                      limit);
-    count_launches(1);
-    ERC_CUDA(cudaGetLastError());
+      ERC_TRY(compact(InducedFlag{g->eu, g->ev, p.nbits}, g->m, edges, (uint32_t*)nullptr,
+                      &p.totals[2], st_m, p.err + 4, abort, limit, s));
   }
   int64_t h_tot[3] = {0, 0, 0};
   unsigned h_err[2] = {0, 0};
