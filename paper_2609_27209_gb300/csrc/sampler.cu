@@ -15,6 +15,8 @@
 // draws and the subgraph's counts: 164 us, 232 us before; 64.3M edges, 6.4M draws: 1.44 ms, 3.95 ms
 // before, with separate passes for weights, draws, marks, induced flags, scans and compactions and
 // two round trips.
+#include <algorithm>
+
 #include "erc_internal.cuh"
 
 namespace erc {
@@ -33,28 +35,46 @@ struct SamplePlan {
   int64_t *E, *Emid, *totals;  // Emid: every SMID-th entry of E; totals: [0] T [1] nodes [2] edges
   uint8_t *nmark, *emark;
   uint32_t* nbits;             // the node marks as bits
-  unsigned long long* status;  // look-back words of the three passes
+  // look-back words of the passes over the weights, the nodes and the edges, side by side
+  unsigned long long *status, *status_n, *status_m;
+  size_t words;
   unsigned* err;  // [0] a probability outside [0, 1]; [1] the abort word; [2..4] the passes' tickets
 };
 
 inline int64_t stile(int64_t count) { return ST * (count < SLARGE ? SIPT_SMALL : SIPT_LARGE); }
 inline int64_t stiles(int64_t count) { return (count + stile(count) - 1) / stile(count); }
-
-// copies of the node marks: at most 16, and 64 MB of them
-inline int mark_copies(int32_t n) {
-  const int64_t c = (int64_t(64) << 20) / n;
-  return c < 1 ? 1 : c > 16 ? 16 : (int)c;
+// The most tiles of a pass over `count` entries or fewer: just below SLARGE entries there are four
+// times as many as from SLARGE on (512 against 128).
+inline int64_t stiles_max(int64_t count) {
+  return std::max(stiles(count), stiles(std::min(count, SLARGE - 1)));
 }
 
-void plan_sample(Arena& a, SamplePlan& p, int64_t count, int32_t n, int64_t m) {
+// copies of the node marks: at most 16, and 64 MB of them
+constexpr int64_t MARK_COPIES = 16, MARK_BYTES = int64_t(64) << 20;
+inline int mark_copies(int32_t n) {
+  return (int)std::max<int64_t>(1, std::min(MARK_COPIES, MARK_BYTES / n));
+}
+// the most bytes of marks of a graph of n nodes or fewer
+inline int64_t mark_bytes_max(int64_t n) {
+  return std::max(n, std::min(MARK_COPIES * n, MARK_BYTES));
+}
+
+// The plan of every call on a graph of n nodes and m edges, drawn by node or by edge.  No array shrinks
+// as n or m grows, so a workspace serves every graph up to the sizes it was reported for.
+void plan_sample(Arena& a, SamplePlan& p, int32_t n, int64_t m) {
+  const int64_t count = std::max<int64_t>(n, m);  // entries drawn from, at most
   p.E = a.take<int64_t>(count);
   p.Emid = a.take<int64_t>(count / SMID + 1);
-  p.nmark = a.take<uint8_t>((size_t)n * mark_copies(n));
+  p.nmark = a.take<uint8_t>(mark_bytes_max(n));
   p.nbits = a.take<uint32_t>((size_t)n / 32 + 1);
   p.emark = a.take<uint8_t>(m > 0 ? m : 1);
   p.totals = a.take<int64_t>(4);
   p.err = a.take<unsigned>(8);
-  p.status = a.take<unsigned long long>(stiles(count) + stiles(n) + stiles(m) + 1);
+  const int64_t w = stiles_max(count), wn = stiles_max(n), wm = stiles_max(m);
+  p.words = (size_t)(w + wn + wm);
+  p.status = a.take<unsigned long long>(p.words);
+  p.status_n = p.status + w;
+  p.status_m = p.status_n + wn;
 }
 
 // W = round(p 2^40) (half up) from the bits of p; p must lie in [0, 1]
@@ -348,7 +368,7 @@ extern "C" size_t erc_sample_workspace_size(int32_t n, int64_t m, int64_t budget
   if (n < 1 || m < 0 || budget < 0) return 0;
   Arena a(nullptr);
   SamplePlan p;
-  plan_sample(a, p, n > m ? n : m, n, m);
+  plan_sample(a, p, n, m);
   return a.used + 256;
 }
 
@@ -372,18 +392,14 @@ extern "C" erc_status erc_sample_subgraph(const erc_graph* g, int32_t kind, cons
   cudaStream_t s = as_stream(stream);
   Arena ar(reinterpret_cast<void*>((reinterpret_cast<uintptr_t>(ws) + 255) & ~uintptr_t(255)));
   SamplePlan p;
-  plan_sample(ar, p, g->n > g->m ? g->n : g->m, g->n, g->m);
+  plan_sample(ar, p, g->n, g->m);
   *n_out = 0;
   *m_out = 0;
   if (count == 0 || budget == 0) return ERC_OK;
   const bool drawn_edges = by_edge && !induced;  // the subgraph keeps the drawn edges alone
   unsigned* abort = p.err + 1;
-  unsigned long long* st_n = p.status + stiles(count);
-  unsigned long long* st_m = st_n + stiles(g->n);
   ERC_CUDA(cudaMemsetAsync(p.err, 0, 8 * sizeof(unsigned), s));
-  ERC_CUDA(cudaMemsetAsync(p.status, 0,
-                           (size_t)(stiles(count) + stiles(g->n) + stiles(g->m)) *
-                               sizeof(unsigned long long), s));
+  ERC_CUDA(cudaMemsetAsync(p.status, 0, p.words * sizeof(*p.status), s));
   const int copies = mark_copies(g->n);
   ERC_CUDA(cudaMemsetAsync(p.nmark, 0, (size_t)g->n * copies, s));
   if (drawn_edges) ERC_CUDA(cudaMemsetAsync(p.emark, 0, (size_t)g->m, s));
@@ -407,14 +423,14 @@ extern "C" erc_status erc_sample_subgraph(const erc_graph* g, int32_t kind, cons
   count_launches(1);
   ERC_CUDA(cudaGetLastError());
   ERC_TRY(compact(CopiesFlag{p.nmark, g->n, copies}, (int64_t)g->n, nodes, p.nbits, &p.totals[1],
-                  st_n, p.err + 3, abort, limit, s));
+                  p.status_n, p.err + 3, abort, limit, s));
   if (g->m > 0) {
     if (drawn_edges)
-      ERC_TRY(compact(MarkedFlag{p.emark}, g->m, edges, (uint32_t*)nullptr, &p.totals[2], st_m,
+      ERC_TRY(compact(MarkedFlag{p.emark}, g->m, edges, (uint32_t*)nullptr, &p.totals[2], p.status_m,
                       p.err + 4, abort, limit, s));
     else
       ERC_TRY(compact(InducedFlag{g->eu, g->ev, p.nbits}, g->m, edges, (uint32_t*)nullptr,
-                      &p.totals[2], st_m, p.err + 4, abort, limit, s));
+                      &p.totals[2], p.status_m, p.err + 4, abort, limit, s));
   }
   int64_t h_tot[3] = {0, 0, 0};
   unsigned h_err[2] = {0, 0};
