@@ -1,5 +1,7 @@
 // sort.cu -- the passes of a stable, deterministic LSD radix sort of (u64 key, u32 value) pairs for
 // the Laplacian build (§3.1.1).
+#include <algorithm>
+
 #include "erc_internal.cuh"
 
 namespace erc {
@@ -219,14 +221,20 @@ void launch_pass(const uint64_t* keys, const uint32_t* vals, uint64_t* keys_out,
 }
 }  // namespace
 
-// tmp: [status: tiles x RS_RADIX][tickets: RS_MAX_PASSES]
+// tmp: [tickets: RS_MAX_PASSES][status: tiles x RS_RADIX].  Just below RS_SMALL keys there are more
+// tiles than from there on (1,024 against 820); the size covers the most tiles of n keys or fewer, so
+// that storage sized for a larger input serves a smaller one.
+static_assert(RS_MAX_PASSES * sizeof(unsigned) % sizeof(unsigned long long) == 0, "status aligned");
+inline size_t sort_tmp_bytes(int64_t tiles) {
+  return RS_MAX_PASSES * sizeof(unsigned) +
+         (size_t)tiles * RS_RADIX * sizeof(unsigned long long);
+}
 size_t radix_sort_temp_bytes(int64_t n) {
-  return (size_t)sort_tiles(n) * RS_RADIX * sizeof(unsigned long long) +
-         RS_MAX_PASSES * sizeof(unsigned);
+  return sort_tmp_bytes(std::max(sort_tiles(n), sort_tiles(std::min(n, RS_SMALL - 1))));
 }
 
 erc_status radix_sort_begin(int64_t n, void* tmp, cudaStream_t s) {
-  ERC_CUDA(cudaMemsetAsync(tmp, 0, radix_sort_temp_bytes(n), s));
+  ERC_CUDA(cudaMemsetAsync(tmp, 0, sort_tmp_bytes(sort_tiles(n)), s));
   return ERC_OK;
 }
 
@@ -235,8 +243,9 @@ erc_status radix_sort_pass(const uint64_t* keys, const uint32_t* vals, uint64_t*
                            const unsigned long long* counts, void* tmp, cudaStream_t s,
                            unsigned* abort) {
   if (n_max <= 0) return ERC_OK;
-  unsigned long long* status = static_cast<unsigned long long*>(tmp);
-  unsigned* ticket = reinterpret_cast<unsigned*>(status + sort_tiles(n_max) * RS_RADIX) + pass;
+  unsigned* ticket = static_cast<unsigned*>(tmp) + pass;
+  unsigned long long* status =
+      reinterpret_cast<unsigned long long*>(static_cast<unsigned*>(tmp) + RS_MAX_PASSES);
   if (sort_small(n_max))
     launch_pass<8>(keys, vals, keys_out, vals_out, n_max, n, shift, pass, counts, status, ticket, s,
                    abort);

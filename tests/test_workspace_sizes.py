@@ -49,3 +49,22 @@ def test_sampler_workspace_of_a_larger_graph_serves_a_smaller_one(size):
     for n in SIZES:
         sizes = [size(n, m, 100) for m in SIZES]
         assert sizes == sorted(sizes), n
+
+
+# both sides of the key count (2^21) where the build's sort takes larger tiles, and sizes between
+INPUTS = [0, 1, 2047, 2049, 500000, (2 << 20) - 4096, (2 << 20) - 1, 2 << 20, (2 << 20) + 1,
+          (2 << 20) + 9000, 2200000, 4194304, 50000000]
+
+
+@pytest.mark.parametrize("call", ["build", "run", "run_host"])
+def test_build_workspace_of_a_larger_graph_serves_a_smaller_one(size, call):
+    L = erc.lib()
+    f = {"build": L.erc_build_laplacian_workspace_size,
+         "run": lambda n, m: L.erc_run_workspace_size(n, m, 64),
+         "run_host": lambda n, m: L.erc_run_host_workspace_size(n, m, 64, 256)}[call]
+    for m in INPUTS:
+        sizes = [f(n, m) for n in SIZES]
+        assert sizes == sorted(sizes), m
+    for n in SIZES:
+        sizes = [f(n, m) for m in INPUTS]
+        assert sizes == sorted(sizes), n
