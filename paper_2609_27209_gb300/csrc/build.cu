@@ -288,7 +288,9 @@ __global__ void __launch_bounds__(BT)
 
 // A running sum in three float32 words, each addition's error carried to the next word exactly: at
 // least 70 bits, where float64 has 53.  GB300 adds float64 at a sixty-fourth of the float32 rate, and
-// the conversions run there too; three words take 13 float32 operations an addend.
+// the conversions run there too; three words take 13 float32 operations an addend.  The addends are
+// positive: once the sum passes the largest float the first word stays infinite, and so is the sum
+// (the other words then hold differences of infinities).
 struct Sum3 {
   float a = 0.f, b = 0.f, c = 0.f;
   __device__ __forceinline__ void add(float x) {
@@ -298,7 +300,9 @@ struct Sum3 {
     b = t.x;
     c = __fadd_rn(c, t.y);
   }
-  __device__ __forceinline__ double value() const { return (double)a + ((double)b + (double)c); }
+  __device__ __forceinline__ double value() const {
+    return isinf(a) ? (double)a : (double)a + ((double)b + (double)c);
+  }
 };
 
 // A row's weights summed to at least float64's precision, rounded once.  Eight lanes a row; a warp's
