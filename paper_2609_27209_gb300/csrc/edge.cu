@@ -288,6 +288,33 @@ __global__ void __launch_bounds__(T)
   }
 }
 
+// A float64 factor f in [0, 1] as three float32 words (all of its 53 bits, scaled to [1, 2] so that no
+// part of a product underflows), and w f to at least 68 bits, rounded once.  The float64 product is
+// rounded to 53 bits first, and GB300 runs it at a sixty-fourth of the float32 rate.
+struct Factor {
+  float a, b, c, back;
+  __device__ explicit Factor(double f) {
+    const int k = f > 0.0 ? ilogb(f) : 0;
+    const double s = ldexp(f, -k);
+    a = (float)s;
+    b = (float)(s - (double)a);
+    c = (float)(s - (double)a - (double)b);
+    back = ldexpf(1.f, k);
+  }
+  __device__ __forceinline__ float times(float w) const {
+    const float p = __fmul_rn(w, a), pe = __fmaf_rn(w, a, -p);
+    const float q = __fmul_rn(w, b), qe = __fmaf_rn(w, b, -q);
+    const float2 s = df_two_sum(pe, q);
+    const float t = __fmaf_rn(w, c, __fadd_rn(qe, s.y));
+    const float2 h = df_norm(p, s.x);
+    // what h.x lacks, rounded to odd: a half of its last place stays distinct from more or less
+    const float2 y = df_two_sum(h.y, t);
+    int bits = __float_as_int(y.x);
+    if (y.y != 0.f && !(bits & 1)) bits += (y.y > 0.f) == (y.x > 0.f) ? 1 : -1;
+    return __fmul_rn(__fadd_rn(h.x, __int_as_float(bits)), back);
+  }
+};
+
 // normalisation: every block forms the three totals from all partials itself (same order in
 // every block), then scales its share of the node and edge weights
 __global__ void k_normalize(const int64_t* __restrict__ row_ptr, const double* __restrict__ qnode,
@@ -321,15 +348,9 @@ __global__ void k_normalize(const int64_t* __restrict__ row_ptr, const double* _
       pr = row_ptr[u + 1] > row_ptr[u] ? uni : 0.0;
     prob_node[u] = (float)pr;
   }
-  // weight times 1 / total, the reciprocal as a float pair: the exact product with its high part and
-  // the product with its low part, rounded once, like the float64 product that GB300 would run at
-  // a sixty-fourth of the float32 rate (64.3M edges: 171 us, 423 us with it)
-  const float2 inv = df_from_double(inv_e);
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += stride) {
-    const float w = edge_weight(kappa[e], kmax);
-    const float p = __fmul_rn(w, inv.x);
-    prob_edge[e] = __fadd_rn(p, __fmaf_rn(w, inv.y, __fmaf_rn(w, inv.x, -p)));
-  }
+  const Factor inv(inv_e);
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += stride)
+    prob_edge[e] = inv.times(edge_weight(kappa[e], kmax));
 }
 
 }  // namespace
