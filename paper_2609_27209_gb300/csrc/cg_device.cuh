@@ -142,6 +142,17 @@ __device__ __forceinline__ Quad ld_quad(const float* p) {
   return quad(L2ONLY ? __ldcg(reinterpret_cast<const float4*>(p)) : ld_f4(p));
 }
 
+// Four columns at p, past L1, where `on`, else v.  A predicated load: a branch would make the lanes of
+// its two sides wait one after the other.
+__device__ __forceinline__ Quad ldcg_quad_if(bool on, const float* p, Quad v) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %3, 0;\n\t"
+      "@q ld.global.cg.v2.u64 {%0, %1}, [%2];\n\t}"
+      : "+l"(v.a), "+l"(v.b)
+      : "l"(p), "r"((unsigned)on));
+  return v;
+}
+
 // The neighbour ids (and weights) of two steps of a group, in shared memory: a step reads four at a
 // time, where lanes that passed each other the ids would take a shuffle for every slot.
 template <int U, bool WEIGHTED>
@@ -162,14 +173,22 @@ struct alignas(16) Slots {
 // neighbour ids -> neighbour rows.  So the chain is taken apart: a step gathers up to U rows at
 // once, and while they are on their way the next step's ids are loaded, which at a row's end are
 // the next row's first, and the bounds of the row after that.  The short last step of a row takes 4,
-// 8 or U slots; those past the end hold the row itself, which is cached and adds exactly zero
-// (loads that are predicated off or replaced by p_u measured up to 13% slower over a solve).
+// 8 or U slots; those past the end hold the row itself.  Through L1 they are loaded, from a cached line,
+// and add exactly zero (128 columns, 150k nodes, 1.5M edges: 130 us, 139 with the loads predicated
+// off).  Past L1 each would be a request to L2, so they are predicated off, and p_u stands for them
+// (20,000 nodes, 160,000 edges, 32 columns: 477 us a solve, 544 with them).
+//
+// The groups of a warp take their steps together, with the longest one's count: left to themselves
+// they drift apart, and a warp then issues, and waits for, each group's gathers in turn (1M nodes, 8M
+// edges of a power law, 32 columns: 383 us an application, 508 before; 1M nodes, 3M edges: 178 us,
+// 237 before).
 template <int LPR, int U, bool WEIGHTED, bool L2ONLY, class Bounds, class Own, class Emit>
 __device__ __forceinline__ void walk_rows(const SpmmArgs& a, const float* __restrict__ srcq,
                                           int gl, unsigned gm, Slots<U, WEIGHTED>& slots,
                                           int nrows, bool on, Bounds&& bounds, Own&& own,
                                           Emit&& emit) {
   constexpr int E = (U + LPR - 1) / LPR;  // ids a lane fetches
+  constexpr bool TOGETHER = LPR < 32;
   const uint32_t ld = (uint32_t)a.ld;
   auto put = [&](int b, const uint32_t(&c)[E], const float(&w)[E]) {
 #pragma unroll
@@ -205,13 +224,13 @@ __device__ __forceinline__ void walk_rows(const SpmmArgs& a, const float* __rest
   __syncwarp(gm);
   Quad pu = {0, 0}, acc = {0, 0};
   bool fresh = true;
-  for (int k = 0; k < nrows;) {
+  for (int k = 0; TOGETHER ? __any_sync(0xffffffffu, k < nrows) : k < nrows;) {
     const bool last = rem <= U;
     fetch(last ? nu : u, last ? nj : j + U, last ? nrem : rem - U, c, w);
     uint32_t bj = 0, bu = 0;
     int brem = -1;
     if (last && k + 2 < nrows) bounds(k + 2, bj, brem, bu);
-    if (fresh) pu = own(u);
+    if (fresh && k < nrows) pu = own(u);
     auto step = [&](auto count) {
       constexpr int N = decltype(count)::value;
       Quad v[N];
@@ -221,7 +240,10 @@ __device__ __forceinline__ void walk_rows(const SpmmArgs& a, const float* __rest
         const uint32_t ids[4] = {id.x, id.y, id.z, id.w};
 #pragma unroll
         for (int r = 0; r < 4; ++r)
-          v[t + r] = on ? ld_quad<L2ONLY>(srcq + (size_t)ids[r] * ld) : Quad{0, 0};
+          if constexpr (L2ONLY)
+            v[t + r] = ldcg_quad_if(on && t + r < rem, srcq + (size_t)ids[r] * ld, pu);
+          else
+            v[t + r] = on ? quad(ld_f4(srcq + (size_t)ids[r] * ld)) : Quad{0, 0};
       }
 #pragma unroll
       for (int t = 0; t < N; t += 4) {
@@ -242,14 +264,15 @@ __device__ __forceinline__ void walk_rows(const SpmmArgs& a, const float* __rest
         }
       }
     };
-    if (rem > 0) {
-      if (rem <= 4) step(ic<4>{});
-      else if (U > 8 && rem <= 8) step(ic<8>{});
+    const int most = TOGETHER ? __reduce_max_sync(0xffffffffu, rem) : rem;
+    if (most > 0) {
+      if (most <= 4) step(ic<4>{});
+      else if (U > 8 && most <= 8) step(ic<8>{});
       else step(ic<U>{});
     }
     put(b ^ 1, c, w);  // last read one step ago, before that step's barrier
     if (last) {
-      if (rem >= 0) emit(k, u, pu, acc);
+      if (rem >= 0) emit(k, u, pu, rem > 0 ? acc : Quad{0, 0});
       acc = Quad{0, 0};
       ++k;
       u = nu;
@@ -264,7 +287,7 @@ __device__ __forceinline__ void walk_rows(const SpmmArgs& a, const float* __rest
     }
     fresh = last;
     b ^= 1;
-    __syncwarp(gm);
+    __syncwarp(TOGETHER ? 0xffffffffu : gm);
   }
 }
 
