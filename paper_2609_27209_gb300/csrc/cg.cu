@@ -1156,8 +1156,9 @@ size_t open_smem(const void* k) {
 // partials, the region shared by the heavy-row slices and the reduction scratch, and the local
 // heavy-row list
 size_t resident_smem(int64_t rows, int ld, bool ps, int hrows) {
-  return 4 * ((ps ? 3 : 2) * (size_t)rows * ld + 2 * (size_t)ld + resident_shared_floats(hrows) +
-              (size_t)rows);
+  const int vpl = ld > 128 ? 2 : 1;  // quads a lane: a group has at most 32 lanes
+  return 4 * ((ps ? 3 : 2) * (size_t)rows * ld + 2 * (size_t)ld +
+              resident_shared_floats(hrows, vpl) + (size_t)rows);
 }
 
 bool resident_plan(const erc_graph* g, int ld, bool pc, int32_t* rb, int32_t* hrows,

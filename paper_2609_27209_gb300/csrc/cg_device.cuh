@@ -152,6 +152,14 @@ __device__ __forceinline__ Quad ldcg_quad_if(bool on, const float* p, Quad v) {
       : "l"(p), "r"((unsigned)on));
   return v;
 }
+__device__ __forceinline__ float4 ldcg_f4_if(bool on, const float* p, float4 v) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %5, 0;\n\t"
+      "@q ld.global.cg.v4.f32 {%0, %1, %2, %3}, [%4];\n\t}"
+      : "+f"(v.x), "+f"(v.y), "+f"(v.z), "+f"(v.w)
+      : "l"(p), "r"((unsigned)on));
+  return v;
+}
 
 // The neighbour ids (and weights) of two steps of a group, in shared memory: a step reads four at a
 // time, where lanes that passed each other the ids would take a shuffle for every slot.
@@ -409,10 +417,59 @@ __device__ __forceinline__ void res_wait(const unsigned* arr, unsigned target, i
   __syncthreads();
 }
 
-// floats of the region that the resident kernel uses for the heavy-row slices, `hrows` rows of one
-// quad per thread, and, after the operator, as the reduction scratch [2 * PT float pairs]
-__host__ __device__ constexpr size_t resident_shared_floats(int hrows) {
-  return 4 * (size_t)PT * (size_t)hrows;
+// floats of the region that the resident kernel uses for the heavy-row slices, `hrows` rows of vpl
+// quads per thread, and, after the operator, as the reduction scratch [2 * PT float pairs]
+__host__ __device__ constexpr size_t resident_shared_floats(int hrows, int vpl) {
+  return 4 * (size_t)PT * (size_t)(hrows * vpl);
+}
+
+// acc[v] += w (p_u - p_v) over the CSR slots [j, j + len) of row u, for the lane's VPL quads of every
+// neighbour at once: rows of more than 128 columns.  The ids pass by shuffles, and 8 / VPL neighbours
+// are in flight.  A walk for each quad passes over the row bounds and ids twice and waits twice
+// (10,000 nodes, 256 columns: 60,000 edges 976 us a solve, 881 with both quads at once, 875 before
+// the walk; 120,000 edges 1,130, 901 and 890).
+template <int LPR, int VPL, bool WEIGHTED>
+__device__ __forceinline__ void gather_wide(const SpmmArgs& a, const float* __restrict__ src, int gl,
+                                            unsigned gm, int nvec, unsigned on, uint32_t j, int len,
+                                            const float4 (&pu)[VPL], float4 (&acc)[VPL]) {
+  constexpr int U = 8 / VPL;
+  for (int jb = 0; jb < len; jb += LPR) {
+    int32_t cidx = 0;
+    float wv = 1.f;
+    if (jb + gl < len) {
+      cidx = __ldg(a.col + (size_t)(j + (uint32_t)(jb + gl)));
+      if (WEIGHTED) wv = __ldg(a.val + (size_t)(j + (uint32_t)(jb + gl)));
+    }
+    const int cnt = min(LPR, len - jb);
+    for (int t = 0; t < cnt; t += U) {
+      int cj[U];
+      float wj[U];
+      float4 pv[U][VPL];
+#pragma unroll
+      for (int k = 0; k < U; ++k) {
+        cj[k] = __shfl_sync(gm, cidx, (t + k) & (LPR - 1), LPR);
+        wj[k] = WEIGHTED ? __shfl_sync(gm, wv, (t + k) & (LPR - 1), LPR) : 1.f;
+        if (t + k >= cnt) wj[k] = 0.f;
+      }
+#pragma unroll
+      for (int k = 0; k < U; ++k)
+#pragma unroll
+        for (int v = 0; v < VPL; ++v) {
+          const int q = gl + LPR * v;
+          pv[k][v] = ldcg_f4_if(q < nvec && t + k < cnt && ((on >> v) & 1u),
+                                src + (size_t)cj[k] * a.ld + 4 * q, pu[v]);
+        }
+#pragma unroll
+      for (int k = 0; k < U; ++k)
+#pragma unroll
+        for (int v = 0; v < VPL; ++v) {
+          acc[v].x = fmaf(wj[k], pu[v].x - pv[k][v].x, acc[v].x);
+          acc[v].y = fmaf(wj[k], pu[v].y - pv[k][v].y, acc[v].y);
+          acc[v].z = fmaf(wj[k], pu[v].z - pv[k][v].z, acc[v].z);
+          acc[v].w = fmaf(wj[k], pu[v].w - pv[k][v].w, acc[v].w);
+        }
+    }
+  }
 }
 
 // o = L_eps s on the rows r0 + i rstep, i < nrows, of s = src (n x ld): o_u = eps s_u +
@@ -429,54 +486,106 @@ __device__ __forceinline__ void block_apply(const SpmmArgs& a, const float* src,
                                             unsigned gm, unsigned on, Own&& own, Emit&& emit) {
   constexpr int GPB = PT / LPR;
   const int nvec = a.ld >> 2;
-  float4* part = reinterpret_cast<float4*>(comb);  // [hrows][PT]
+  float4* part = reinterpret_cast<float4*>(comb);  // [hrows][VPL][PT]
+  if constexpr (VPL > 1) {
+    auto load = [&](int64_t u, float4(&pu)[VPL], float4(&acc)[VPL]) {
 #pragma unroll
-  for (int v = 0; v < VPL; ++v) {
-    const int q = gl + LPR * v;
-    const bool valid = q < nvec, lane_on = valid && ((on >> v) & 1u);
-    const float* srcq = src + 4 * (valid ? q : 0);
-    auto own_quad = [&](uint32_t u) { return lane_on ? quad(own((int64_t)u, v)) : Quad{0, 0}; };
+      for (int v = 0; v < VPL; ++v) {
+        pu[v] = gl + LPR * v < nvec && ((on >> v) & 1u) ? own(u, v) : f4_zero();
+        acc[v] = f4_zero();
+      }
+    };
+    auto give = [&](int i, int64_t u, const float4(&pu)[VPL], const float4(&acc)[VPL]) {
+#pragma unroll
+      for (int v = 0; v < VPL; ++v)
+        if (gl + LPR * v < nvec)
+          emit(i, u, v, pu[v], unquad(apply_quad(a.eps, quad(pu[v]), quad(acc[v]))));
+    };
+    float4 pu[VPL], acc[VPL];
     for (int hb = 0; hb < nh; hb += hrows) {
       const int cnt = min(hrows, nh - hb);
-      walk_rows<LPR, RUB<LPR>, WEIGHTED, true>(
-          a, srcq, gl, gm, slots, cnt, lane_on,
-          [&](int k, uint32_t& j, int& len, uint32_t& u) {
-            u = (uint32_t)(r0 + hv[hb + k] * rstep);
-            heavy_slice(a.row_ptr, u, gi, GPB, j, len);
-          },
-          own_quad,
-          [&](int k, uint32_t, Quad, Quad acc) { part[k * PT + threadIdx.x] = unquad(acc); });
+      for (int k = 0; k < cnt; ++k) {
+        const int64_t u = r0 + hv[hb + k] * rstep;
+        uint32_t j;
+        int len;
+        heavy_slice(a.row_ptr, u, gi, GPB, j, len);
+        load(u, pu, acc);
+        gather_wide<LPR, VPL, WEIGHTED>(a, src, gl, gm, nvec, on, j, len, pu, acc);
+#pragma unroll
+        for (int v = 0; v < VPL; ++v) part[(k * VPL + v) * PT + threadIdx.x] = acc[v];
+      }
       __syncthreads();
       for (int k = gi; k < cnt; k += GPB) {
         const int i = hv[hb + k];
-        const int64_t u = r0 + i * rstep;
-        const Quad pu = own_quad((uint32_t)u);
-        Quad sum = {0, 0};
-#pragma unroll 8
-        for (int g = 0; g < GPB; ++g) {
-          const Quad x = quad(part[k * PT + g * LPR + gl]);
-          sum.a = add2(sum.a, x.a);
-          sum.b = add2(sum.b, x.b);
-        }
-        if (valid) emit(i, u, v, unquad(pu), unquad(apply_quad(a.eps, pu, sum)));
+        load(r0 + i * rstep, pu, acc);
+#pragma unroll
+        for (int v = 0; v < VPL; ++v)
+#pragma unroll 4
+          for (int g = 0; g < GPB; ++g) {
+            const float4 x = part[(k * VPL + v) * PT + g * LPR + gl];
+            acc[v].x += x.x;
+            acc[v].y += x.y;
+            acc[v].z += x.z;
+            acc[v].w += x.w;
+          }
+        give(i, r0 + i * rstep, pu, acc);
       }
       __syncthreads();
     }
-    const int mine = nrows > gi ? (nrows - gi + GPB - 1) / GPB : 0;
+    for (int i = gi; i < nrows; i += GPB) {
+      const int64_t u = r0 + i * rstep;
+      uint32_t j, len;
+      row_slots(a.row_ptr, u, j, len);
+      if (len > (uint32_t)a.H) continue;
+      load(u, pu, acc);
+      gather_wide<LPR, VPL, WEIGHTED>(a, src, gl, gm, nvec, on, j, (int)len, pu, acc);
+      give(i, u, pu, acc);
+    }
+    return;
+  }
+  const bool valid = gl < nvec, lane_on = valid && (on & 1u);
+  const float* srcq = src + 4 * (valid ? gl : 0);
+  auto own_quad = [&](uint32_t u) { return lane_on ? quad(own((int64_t)u, 0)) : Quad{0, 0}; };
+  for (int hb = 0; hb < nh; hb += hrows) {
+    const int cnt = min(hrows, nh - hb);
     walk_rows<LPR, RUB<LPR>, WEIGHTED, true>(
-        a, srcq, gl, gm, slots, mine, lane_on,
+        a, srcq, gl, gm, slots, cnt, lane_on,
         [&](int k, uint32_t& j, int& len, uint32_t& u) {
-          u = (uint32_t)(r0 + (gi + k * GPB) * rstep);
-          uint32_t n;
-          row_slots(a.row_ptr, u, j, n);
-          len = n > (uint32_t)a.H ? -1 : (int)n;
+          u = (uint32_t)(r0 + hv[hb + k] * rstep);
+          heavy_slice(a.row_ptr, u, gi, GPB, j, len);
         },
         own_quad,
-        [&](int k, uint32_t u, Quad pu, Quad acc) {
-          if (valid)
-            emit(gi + k * GPB, (int64_t)u, v, unquad(pu), unquad(apply_quad(a.eps, pu, acc)));
-        });
+        [&](int k, uint32_t, Quad, Quad acc) { part[k * PT + threadIdx.x] = unquad(acc); });
+    __syncthreads();
+    for (int k = gi; k < cnt; k += GPB) {
+      const int i = hv[hb + k];
+      const int64_t u = r0 + i * rstep;
+      const Quad pu = own_quad((uint32_t)u);
+      Quad sum = {0, 0};
+#pragma unroll 8
+      for (int g = 0; g < GPB; ++g) {
+        const Quad x = quad(part[k * PT + g * LPR + gl]);
+        sum.a = add2(sum.a, x.a);
+        sum.b = add2(sum.b, x.b);
+      }
+      if (valid) emit(i, u, 0, unquad(pu), unquad(apply_quad(a.eps, pu, sum)));
+    }
+    __syncthreads();
   }
+  const int mine = nrows > gi ? (nrows - gi + GPB - 1) / GPB : 0;
+  walk_rows<LPR, RUB<LPR>, WEIGHTED, true>(
+      a, srcq, gl, gm, slots, mine, lane_on,
+      [&](int k, uint32_t& j, int& len, uint32_t& u) {
+        u = (uint32_t)(r0 + (gi + k * GPB) * rstep);
+        uint32_t n;
+        row_slots(a.row_ptr, u, j, n);
+        len = n > (uint32_t)a.H ? -1 : (int)n;
+      },
+      own_quad,
+      [&](int k, uint32_t u, Quad pu, Quad acc) {
+        if (valid)
+          emit(gi + k * GPB, (int64_t)u, 0, unquad(pu), unquad(apply_quad(a.eps, pu, acc)));
+      });
 }
 
 // the block's part of a grid-wide column sum: publish the block's partials (row blockIdx.x of
@@ -514,7 +623,7 @@ __global__ void __launch_bounds__(PT, 1) k_cg_resident(ResArgs ra) {
   // the block gathers
   float* comb = reinterpret_cast<float*>(sbuf + ld);
   float2* scratch = sbuf + ld;
-  int* hv = reinterpret_cast<int*>(comb + resident_shared_floats(ra.hrows));
+  int* hv = reinterpret_cast<int*>(comb + resident_shared_floats(ra.hrows, VPL));
   // block partials, one region per reduction kind so that no block overwrites partials another
   // block may still be summing: [G][ld] each
   float2* part_pap = a.cr.part1;
