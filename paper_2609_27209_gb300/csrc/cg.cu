@@ -1169,7 +1169,7 @@ bool resident_plan(const erc_graph* g, int ld, bool pc, int32_t* rb, int32_t* hr
   for (int ps = 1; ps >= 0; --ps) {  // p in shared memory when it fits
     const void* k = resident_kernel(nvec, g->val != nullptr, ps, pc);
     if (!k) return false;
-    int hr = 8;  // heavy rows between two barriers: as many as the memory left over holds
+    int hr = HROWS_MAX;  // heavy rows between two barriers: as many as the memory left over holds
     while (hr > 1 && resident_smem(rows, ld, ps, hr) > open_smem(k)) hr /= 2;
     const size_t bytes = resident_smem(rows, ld, ps, hr);
     if (bytes > open_smem(k)) continue;

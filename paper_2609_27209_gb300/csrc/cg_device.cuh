@@ -161,12 +161,16 @@ __device__ __forceinline__ float4 ldcg_f4_if(bool on, const float* p, float4 v) 
   return v;
 }
 
-// The neighbour ids (and weights) of two steps of a group, in shared memory: a step reads four at a
-// time, where lanes that passed each other the ids would take a shuffle for every slot.
+// The neighbour ids (and weights) of a group's step, in shared memory: the step reads four at a time,
+// where lanes that passed each other the ids would take a shuffle for every slot.
 template <int U, bool WEIGHTED>
 struct alignas(16) Slots {
-  uint32_t id[2][U];
-  float w[WEIGHTED ? 2 : 1][WEIGHTED ? U : 4];
+  uint32_t id[U];
+  float w[U];
+};
+template <int U>
+struct alignas(16) Slots<U, false> {
+  uint32_t id[U];
 };
 
 // A group of LPR lanes walks a list of `nrows` rows, four columns a lane: row k's sum over its
@@ -198,13 +202,13 @@ __device__ __forceinline__ void walk_rows(const SpmmArgs& a, const float* __rest
   constexpr int E = (U + LPR - 1) / LPR;  // ids a lane fetches
   constexpr bool TOGETHER = LPR < 32;
   const uint32_t ld = (uint32_t)a.ld;
-  auto put = [&](int b, const uint32_t(&c)[E], const float(&w)[E]) {
+  auto put = [&](const uint32_t(&c)[E], const float(&w)[E]) {
 #pragma unroll
     for (int e = 0; e < E; ++e) {
       const int k = gl + e * LPR;
       if (U % LPR != 0 && k >= U) continue;
-      slots.id[b][k] = c[e];
-      if (WEIGHTED) slots.w[b][k] = w[e];
+      slots.id[k] = c[e];
+      if constexpr (WEIGHTED) slots.w[k] = w[e];
     }
   };
   auto fetch = [&](uint32_t u, uint32_t j, int rem, uint32_t(&c)[E], float(&w)[E]) {
@@ -225,10 +229,9 @@ __device__ __forceinline__ void walk_rows(const SpmmArgs& a, const float* __rest
   if (nrows > 1) bounds(1, nj, nrem, nu);
   uint32_t c[E];
   float w[E];
-  int b = 0;  // the buffer that holds this step's slots
   fetch(u, j, rem, c, w);
   __syncwarp(gm);  // the group is done with the slots of an earlier walk
-  put(0, c, w);
+  put(c, w);
   __syncwarp(gm);
   Quad pu = {0, 0}, acc = {0, 0};
   bool fresh = true;
@@ -244,7 +247,7 @@ __device__ __forceinline__ void walk_rows(const SpmmArgs& a, const float* __rest
       Quad v[N];
 #pragma unroll
       for (int t = 0; t < N; t += 4) {
-        const uint4 id = *reinterpret_cast<const uint4*>(&slots.id[b][t]);
+        const uint4 id = *reinterpret_cast<const uint4*>(&slots.id[t]);
         const uint32_t ids[4] = {id.x, id.y, id.z, id.w};
 #pragma unroll
         for (int r = 0; r < 4; ++r)
@@ -256,7 +259,7 @@ __device__ __forceinline__ void walk_rows(const SpmmArgs& a, const float* __rest
 #pragma unroll
       for (int t = 0; t < N; t += 4) {
         float4 wq = make_float4(1.f, 1.f, 1.f, 1.f);
-        if constexpr (WEIGHTED) wq = *reinterpret_cast<const float4*>(&slots.w[b][t]);
+        if constexpr (WEIGHTED) wq = *reinterpret_cast<const float4*>(&slots.w[t]);
         const float ws[4] = {wq.x, wq.y, wq.z, wq.w};
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
@@ -278,7 +281,8 @@ __device__ __forceinline__ void walk_rows(const SpmmArgs& a, const float* __rest
       else if (U > 8 && most <= 8) step(ic<8>{});
       else step(ic<U>{});
     }
-    put(b ^ 1, c, w);  // last read one step ago, before that step's barrier
+    __syncwarp(TOGETHER ? 0xffffffffu : gm);  // the group is done with this step's slots
+    put(c, w);
     if (last) {
       if (rem >= 0) emit(k, u, pu, rem > 0 ? acc : Quad{0, 0});
       acc = Quad{0, 0};
@@ -294,7 +298,6 @@ __device__ __forceinline__ void walk_rows(const SpmmArgs& a, const float* __rest
       rem -= U;
     }
     fresh = last;
-    b ^= 1;
     __syncwarp(TOGETHER ? 0xffffffffu : gm);
   }
 }
@@ -379,9 +382,10 @@ constexpr int PT = 512;
 constexpr int PWARPS = PT / 32;
 constexpr int PCH = 64;
 constexpr int RMAXLD = 256;  // widest row block the resident kernel takes (64 float4)
+constexpr int HROWS_MAX = 8;
 constexpr int RU = 2;  // float4 loads per lane in flight in phases B and C
-// neighbour rows in flight per row group in the gathers (fewer for the narrowest rows, whose many
-// groups would otherwise take 32 KB of shared memory for their slots)
+// neighbour rows in flight per row group in the gathers (fewer for the narrowest rows, so that no
+// shape's slots take more than 8 KB: the memory left bounds the rows that the solver can take)
 template <int LPR>
 constexpr int RUB = LPR == 4 ? 8 : 16;
 
@@ -556,15 +560,17 @@ __device__ __forceinline__ void block_apply(const SpmmArgs& a, const float* src,
         },
         own_quad,
         [&](int k, uint32_t, Quad, Quad acc) { part[k * PT + threadIdx.x] = unquad(acc); });
+    // a group adds the slices of at most one row; its p is on the way meanwhile
+    static_assert(GPB >= HROWS_MAX, "a group a heavy row");
+    const int i = gi < cnt ? hv[hb + gi] : 0;
+    const int64_t u = r0 + i * rstep;
+    const Quad pu = gi < cnt ? own_quad((uint32_t)u) : Quad{0, 0};
     __syncthreads();
-    for (int k = gi; k < cnt; k += GPB) {
-      const int i = hv[hb + k];
-      const int64_t u = r0 + i * rstep;
-      const Quad pu = own_quad((uint32_t)u);
+    if (gi < cnt) {
       Quad sum = {0, 0};
 #pragma unroll 8
       for (int g = 0; g < GPB; ++g) {
-        const Quad x = quad(part[k * PT + g * LPR + gl]);
+        const Quad x = quad(part[gi * PT + g * LPR + gl]);
         sum.a = add2(sum.a, x.a);
         sum.b = add2(sum.b, x.b);
       }
@@ -636,14 +642,15 @@ __global__ void __launch_bounds__(PT, 1) k_cg_resident(ResArgs ra) {
   float2* part_res = a.cr.part1 + 4 * (size_t)G * ld;
   unsigned* arrivals = va.gen;
   // per-column CG state, the same in every block
-  __shared__ float2 s_rr[RMAXLD], s_yy[RMAXLD];  // float pairs; s_rr holds r.z with PC
-  __shared__ float2 s_rz[PC ? RMAXLD : 1];        // the new r.z of phase B (PC)
-  __shared__ __align__(16) float s_alpha[RMAXLD], s_beta[RMAXLD];
-  __shared__ __align__(16) int s_active[RMAXLD];
-  __shared__ int s_iters[RMAXLD], s_conv[RMAXLD];
+  constexpr int MAXC = 4 * LPR * VPL;
+  __shared__ float2 s_rr[MAXC], s_yy[MAXC];  // float pairs; s_rr holds r.z with PC
+  __shared__ float2 s_rz[PC ? MAXC : 1];        // the new r.z of phase B (PC)
+  __shared__ __align__(16) float s_alpha[MAXC], s_beta[MAXC];
+  __shared__ __align__(16) int s_active[MAXC];
+  __shared__ int s_iters[MAXC], s_conv[MAXC];
   __shared__ int s_nh, s_wcnt[PWARPS];
   __shared__ unsigned s_most;
-  __shared__ Slots<RUB<LPR>, WEIGHTED> slots[GPB];
+  __shared__ Slots<RUB<LPR>, WEIGHTED> slots[VPL == 1 ? GPB : 1];  // the wide rows have none
 
   // ---- which rows the block gathers in A: its own, or dealt ones where the own ranges are so
   // uneven that the largest would cost more than 4 us an iteration over the mean.  A gathered
@@ -788,7 +795,7 @@ __global__ void __launch_bounds__(PT, 1) k_cg_resident(ResArgs ra) {
 #pragma unroll
       for (int t = 0; t < 4; ++t) dot[v][t] = make_float2(0.f, 0.f);
     block_apply<LPR, VPL, WEIGHTED>(
-        a, a.P, g0, gstep, grows, hv, nh, ra.hrows, comb, slots[gi], gl, gi, gm, on,
+        a, a.P, g0, gstep, grows, hv, nh, ra.hrows, comb, slots[VPL == 1 ? gi : 0], gl, gi, gm, on,
         [&](int64_t u, int v) {
           const int q = gl + LPR * v;
           return PS && !deal ? reinterpret_cast<const float4*>(ps + (size_t)(u - r0) * ld)[q]
@@ -982,7 +989,7 @@ __global__ void __launch_bounds__(PT, 1) k_cg_resident(ResArgs ra) {
 #pragma unroll
     for (int t = 0; t < 4; ++t) dot[v][t] = make_float2(0.f, 0.f);
   block_apply<LPR, VPL, WEIGHTED>(
-      a, va.X, g0, gstep, grows, hv, nh, ra.hrows, comb, slots[gi], gl, gi, gm, ~0u,
+      a, va.X, g0, gstep, grows, hv, nh, ra.hrows, comb, slots[VPL == 1 ? gi : 0], gl, gi, gm, ~0u,
       [&](int64_t u, int v) { return ldcg_f4(va.X + (size_t)u * ld + 4 * (gl + LPR * v)); },
       [&](int, int64_t u, int v, float4, float4 o) {
         const int q = gl + LPR * v, cb = 4 * q;
