@@ -262,7 +262,8 @@ erc_status erc_sampling_probs_noalloc(const erc_graph* g, const float* kappa, fl
  * Out: nodes [capacity n] ascending distinct node ids, *n_out (host); edges [capacity m]
  *   ascending canonical edge ids, *m_out (host).  Deterministic.
  * Errors: INVALID_ARG for a probability outside [0, 1] or all weights rounding to zero;
- *   CAPACITY if ws_bytes < erc_sample_workspace_size(n, m, budget).  Synchronises s.
+ *   CAPACITY if ws_bytes < erc_sample_workspace_size(n, m, budget); nodes and edges are then left
+ *   as they were.  Synchronises s.
  * ------------------------------------------------------------------------------------------- */
 enum { ERC_SAMPLE_NODES = 0, ERC_SAMPLE_EDGES = 1 };
 size_t erc_sample_workspace_size(int32_t n, int64_t m, int64_t budget);

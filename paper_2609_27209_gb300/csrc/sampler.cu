@@ -38,8 +38,12 @@ struct SamplePlan {
   // look-back words of the passes over the weights, the nodes and the edges, side by side
   unsigned long long *status, *status_n, *status_m;
   size_t words;
-  unsigned* err;  // [0] a probability outside [0, 1]; [1] the abort word; [2..4] the passes' tickets
+  unsigned* err;  // [0] the abort word; [1..3] the passes' tickets
 };
+// Bits of the abort word.  Once one is set the passes that follow write nothing: a call that reports
+// an error leaves its outputs alone.  (A word of its own for each reason, read by every block of the
+// compactions, took 3% to 12% of a call.)
+constexpr unsigned WAIT_RAN_OUT = 1, BAD_PROB = 2, NO_WEIGHT = 4;  // tile_prefix sets the first
 
 inline int64_t stile(int64_t count) { return ST * (count < SLARGE ? SIPT_SMALL : SIPT_LARGE); }
 inline int64_t stiles(int64_t count) { return (count + stile(count) - 1) / stile(count); }
@@ -92,7 +96,7 @@ __device__ __forceinline__ uint64_t fixed_weight(float p, bool& bad) {
   return shift > -40 ? (mant + (1ull << (-shift - 1))) >> (-shift) : 0;
 }
 
-// the block's tile of a pass, or -1 once a wait of the call has given up
+// the block's tile of a pass, or -1 once the call has failed
 __device__ __forceinline__ int64_t claim_tile(unsigned* ticket, const unsigned* abort) {
   __shared__ unsigned s_tile;
   if (threadIdx.x == 0) s_tile = aborted(abort) ? 0xffffffffu : atomicAdd(ticket, 1u);
@@ -106,10 +110,11 @@ template <int SIPT>
 __global__ void __launch_bounds__(ST)
     k_weight_scan(const float* __restrict__ prob, int64_t count, bool vec, int64_t* __restrict__ E,
                   int64_t* __restrict__ Emid, int64_t* __restrict__ total,
-                  unsigned long long* status, unsigned* err, unsigned spin_limit) {
+                  unsigned long long* status, unsigned* ticket, unsigned* abort,
+                  unsigned spin_limit) {
   constexpr int64_t STILE = ST * SIPT;
   __shared__ unsigned long long s_warp[SWARPS], s_prefix, s_total;
-  const int64_t t = claim_tile(err + 2, err + 1);
+  const int64_t t = claim_tile(ticket, abort);
   if (t < 0) return;
   constexpr int ROUNDS = SIPT / 4;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -136,7 +141,7 @@ __global__ void __launch_bounds__(ST)
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
   if (lane == 0) s_warp[warp] = sum;
-  if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(err, 1u);
+  if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(abort, BAD_PROB);
   if (warp == 0) {
     const unsigned long long w = lane < SWARPS ? s_warp[lane] : 0;
     unsigned long long inc = w;
@@ -147,7 +152,7 @@ __global__ void __launch_bounds__(ST)
     }
     if (lane < SWARPS) s_warp[lane] = inc - w;
     const unsigned long long tot = __shfl_sync(0xffffffffu, inc, SWARPS - 1);
-    const unsigned long long prefix = tile_prefix(status, t, tot, spin_limit, err + 1);
+    const unsigned long long prefix = tile_prefix(status, t, tot, spin_limit, abort);
     if (lane == 0) {
       s_prefix = prefix;
       s_total = prefix + tot;
@@ -179,7 +184,10 @@ __global__ void __launch_bounds__(ST)
     if (lane % (SMID / 4) == 0 && i < count) Emid[i / SMID] = (int64_t)e0;
     run += __shfl_sync(0xffffffffu, inc, 31);
   }
-  if ((t + 1) * STILE >= count && threadIdx.x == 0) *total = (int64_t)s_total;
+  if ((t + 1) * STILE >= count && threadIdx.x == 0) {
+    *total = (int64_t)s_total;
+    if (s_total == 0) atomicOr(abort, NO_WEIGHT);
+  }
 }
 
 // draw k: the largest i with E_i <= floor(x_k T / 2^64), found in the scan's tiles (their final status
@@ -397,49 +405,53 @@ extern "C" erc_status erc_sample_subgraph(const erc_graph* g, int32_t kind, cons
   *m_out = 0;
   if (count == 0 || budget == 0) return ERC_OK;
   const bool drawn_edges = by_edge && !induced;  // the subgraph keeps the drawn edges alone
-  unsigned* abort = p.err + 1;
+  unsigned* abort = p.err;
   ERC_CUDA(cudaMemsetAsync(p.err, 0, 8 * sizeof(unsigned), s));
   ERC_CUDA(cudaMemsetAsync(p.status, 0, p.words * sizeof(*p.status), s));
   const int copies = mark_copies(g->n);
   ERC_CUDA(cudaMemsetAsync(p.nmark, 0, (size_t)g->n * copies, s));
   if (drawn_edges) ERC_CUDA(cudaMemsetAsync(p.emark, 0, (size_t)g->m, s));
-  // Nothing is read back before the end: a probability outside [0, 1] counts as zero, with a total of
-  // zero every draw is the last index, and the prefixes are only ever below their true values when
-  // a bounded wait gives up, so every index stays in range; the host then reports the error.
+  // Nothing is read back before the end.  A wait that gives up within a compaction leaves its output
+  // incomplete; the prefixes are then below their true values, so every index stays in range.
   const unsigned limit = wait_limit(LOOKBACK_SPINS);
   const bool vec = (reinterpret_cast<uintptr_t>(prob) & 15) == 0;
   if (count < SLARGE)
     k_weight_scan<SIPT_SMALL><<<(unsigned)stiles(count), ST, 0, s>>>(
-        prob, count, vec, p.E, p.Emid, &p.totals[0], p.status, p.err, limit);
+        prob, count, vec, p.E, p.Emid, &p.totals[0], p.status, p.err + 1, abort, limit);
   else
     k_weight_scan<SIPT_LARGE><<<(unsigned)stiles(count), ST, 0, s>>>(
-        prob, count, vec, p.E, p.Emid, &p.totals[0], p.status, p.err, limit);
+        prob, count, vec, p.E, p.Emid, &p.totals[0], p.status, p.err + 1, abort, limit);
   count_launches(1);
   ERC_CUDA(cudaGetLastError());
   const uint2 key = make_uint2((uint32_t)(seed & 0xffffffffu), (uint32_t)(seed >> 32));
-  k_draw<<<grid_for(budget, ST), ST, 0, s>>>(p.E, p.Emid, count, stile(count), p.status, p.totals, budget, key, first_draw,
-                                             by_edge ? 1u : 0u, g->eu, g->ev, p.nmark, g->n,
-                                             copies, drawn_edges ? p.emark : nullptr, abort);
+  k_draw<<<grid_for(budget, ST), ST, 0, s>>>(
+      p.E, p.Emid, count, stile(count), p.status, p.totals, budget, key, first_draw,
+      by_edge ? 1u : 0u, g->eu, g->ev, p.nmark, g->n, copies, drawn_edges ? p.emark : nullptr,
+      abort);
   count_launches(1);
   ERC_CUDA(cudaGetLastError());
   ERC_TRY(compact(CopiesFlag{p.nmark, g->n, copies}, (int64_t)g->n, nodes, p.nbits, &p.totals[1],
-                  p.status_n, p.err + 3, abort, limit, s));
+                  p.status_n, p.err + 2, abort, limit, s));
   if (g->m > 0) {
     if (drawn_edges)
       ERC_TRY(compact(MarkedFlag{p.emark}, g->m, edges, (uint32_t*)nullptr, &p.totals[2], p.status_m,
-                      p.err + 4, abort, limit, s));
+                      p.err + 3, abort, limit, s));
     else
       ERC_TRY(compact(InducedFlag{g->eu, g->ev, p.nbits}, g->m, edges, (uint32_t*)nullptr,
-                      &p.totals[2], p.status_m, p.err + 4, abort, limit, s));
+                      &p.totals[2], p.status_m, p.err + 3, abort, limit, s));
   }
   int64_t h_tot[3] = {0, 0, 0};
-  unsigned h_err[2] = {0, 0};
+  unsigned h_err = 0;
   ERC_CUDA(cudaMemcpyAsync(h_tot, p.totals, 3 * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-  ERC_CUDA(cudaMemcpyAsync(h_err, p.err, 2 * sizeof(unsigned), cudaMemcpyDeviceToHost, s));
+  ERC_CUDA(cudaMemcpyAsync(&h_err, abort, sizeof h_err, cudaMemcpyDeviceToHost, s));
   ERC_CUDA(cudaStreamSynchronize(s));
-  if (h_err[0]) return set_error(ERC_ERR_INVALID_ARG, "probabilities must lie in [0, 1]");
-  if (h_err[1]) return set_error(ERC_ERR_TIMEOUT, "a bounded wait in the sampler's scans ran out");
-  if (h_tot[0] == 0) return set_error(ERC_ERR_INVALID_ARG, "every probability rounds to zero");
+  // a probability out of range stops other tiles' waits, and a scan that gave up may total zero
+  if (h_err & BAD_PROB)
+    return set_error(ERC_ERR_INVALID_ARG, "probabilities must lie in [0, 1]");
+  if (h_err & WAIT_RAN_OUT)
+    return set_error(ERC_ERR_TIMEOUT, "a bounded wait in the sampler's scans ran out");
+  if (h_err & NO_WEIGHT)
+    return set_error(ERC_ERR_INVALID_ARG, "every probability rounds to zero");
   *n_out = (int32_t)h_tot[1];
   *m_out = g->m > 0 ? h_tot[2] : 0;
   return ERC_OK;
