@@ -27,12 +27,17 @@ __device__ __forceinline__ float4 ld_f4(const float* p) {
 // edges a step and four blocks an SM: 2.45M nodes, 64.3M edges, 128 columns, distances to
 // probabilities: 7.73 -> 6.81 ms (eight edges 7.46 with three blocks and 8.01 with four; five blocks
 // 7.96), with both rows loaded for every edge before.
+// Wider rows, with the blocks an SM that their registers allow; from 257 columns on every lane loads the
+// ids itself, because a group is a warp there and the shuffles are on the path to the first row.
+// 1M nodes, 8M edges, 192 columns: 0.95 ms (1.04 with both rows for every edge, 1.16 with three
+// blocks); 20,000 nodes, 200,000 edges, 384 columns: 43.4 us (43.5, and 49.1 with one edge a step in two
+// blocks and ids by shuffles).
 template <int LPR, int VPL>
-__global__ void __launch_bounds__(T, VPL == 1 ? 4 : VPL == 2 ? 3 : 2)
+__global__ void __launch_bounds__(T, VPL <= 2 ? 4 : VPL == 4 ? 3 : 2)
     k_edge_resistance(const int32_t* __restrict__ eu, const int32_t* __restrict__ ev, int64_t m,
                       const float* __restrict__ X, int32_t ld, int32_t kc, float* __restrict__ R) {
   constexpr int SEG = 32;
-  constexpr int EB = VPL <= 4 ? 4 / VPL : 1;
+  constexpr int EB = VPL == 1 ? 4 : VPL <= 4 ? 2 : 1;
   static_assert(EB <= LPR && SEG % EB == 0, "a lane an edge");
   const int gl = threadIdx.x & (LPR - 1);
   const int gpb = T / LPR;
@@ -49,8 +54,14 @@ __global__ void __launch_bounds__(T, VPL == 1 ? 4 : VPL == 2 ? 3 : 2)
       const int32_t lu = __ldg(eu + e), lv = __ldg(ev + e);
 #pragma unroll
       for (int k = 0; k < EB; ++k) {
-        u[k] = __shfl_sync(gm, lu, k, LPR);
-        v[k] = __shfl_sync(gm, lv, k, LPR);
+        if (VPL >= 4) {
+          const int64_t ek = min(eb + k, e1 - 1);
+          u[k] = __ldg(eu + ek);
+          v[k] = __ldg(ev + ek);
+        } else {
+          u[k] = __shfl_sync(gm, lu, k, LPR);
+          v[k] = __shfl_sync(gm, lv, k, LPR);
+        }
       }
       const bool writes = gl < EB && eb + gl < e1;
       const float rold = writes ? R[eb + gl] : 0.f;
