@@ -221,13 +221,13 @@ void launch_pass(const uint64_t* keys, const uint32_t* vals, uint64_t* keys_out,
 }
 }  // namespace
 
-// tmp: [tickets: RS_MAX_PASSES][status: tiles x RS_RADIX].  Just below RS_SMALL keys there are more
-// tiles than from there on (1,024 against 820); the size covers the most tiles of n keys or fewer, so
-// that storage sized for a larger input serves a smaller one.
-static_assert(RS_MAX_PASSES * sizeof(unsigned) % sizeof(unsigned long long) == 0, "status aligned");
+// tmp: [tickets][status: tiles x RS_RADIX].  Just below RS_SMALL keys there are more tiles than from
+// there on (1,024 against 820); the size covers the most tiles of n keys or fewer, so that storage
+// sized for a larger input serves a smaller one.  A tile's status words start on a line.
+constexpr size_t RS_TICKETS = 256;  // bytes
+static_assert(RS_MAX_PASSES * sizeof(unsigned) <= RS_TICKETS, "a ticket a pass");
 inline size_t sort_tmp_bytes(int64_t tiles) {
-  return RS_MAX_PASSES * sizeof(unsigned) +
-         (size_t)tiles * RS_RADIX * sizeof(unsigned long long);
+  return RS_TICKETS + (size_t)tiles * RS_RADIX * sizeof(unsigned long long);
 }
 size_t radix_sort_temp_bytes(int64_t n) {
   return sort_tmp_bytes(std::max(sort_tiles(n), sort_tiles(std::min(n, RS_SMALL - 1))));
@@ -245,7 +245,7 @@ erc_status radix_sort_pass(const uint64_t* keys, const uint32_t* vals, uint64_t*
   if (n_max <= 0) return ERC_OK;
   unsigned* ticket = static_cast<unsigned*>(tmp) + pass;
   unsigned long long* status =
-      reinterpret_cast<unsigned long long*>(static_cast<unsigned*>(tmp) + RS_MAX_PASSES);
+      reinterpret_cast<unsigned long long*>(static_cast<char*>(tmp) + RS_TICKETS);
   if (sort_small(n_max))
     launch_pass<8>(keys, vals, keys_out, vals_out, n_max, n, shift, pass, counts, status, ticket, s,
                    abort);
