@@ -84,7 +84,7 @@ __global__ void __launch_bounds__(T, 2) k_spmm(const __grid_constant__ SpmmArgs 
   constexpr int GPB = T / LPR;  // groups per block
   __shared__ float4 part[HB][T];  // heavy-row slices, then the dot products' scratch
   __shared__ float2 sbuf[MAX_LD];
-  __shared__ Slots<U_SPMM, WEIGHTED> slots[GPB];
+  __shared__ Slots<U_SPMM, WEIGHTED, 2> slots[GPB];
   const int gl = threadIdx.x & (LPR - 1);
   const int gi = threadIdx.x / LPR;
   const int nvec = a.ld >> 2;

@@ -162,15 +162,17 @@ __device__ __forceinline__ float4 ldcg_f4_if(bool on, const float* p, float4 v) 
 }
 
 // The neighbour ids (and weights) of a group's step, in shared memory: the step reads four at a time,
-// where lanes that passed each other the ids would take a shuffle for every slot.
-template <int U, bool WEIGHTED>
+// where lanes that passed each other the ids would take a shuffle for every slot.  With NB = 2 the
+// next step's are put beside this step's; with one set, in the resident solver, whose rows compete for
+// the memory, they wait until the group is done with them.
+template <int U, bool WEIGHTED, int NB>
 struct alignas(16) Slots {
-  uint32_t id[U];
-  float w[U];
+  uint32_t id[NB][U];
+  float w[NB][U];
 };
-template <int U>
-struct alignas(16) Slots<U, false> {
-  uint32_t id[U];
+template <int U, int NB>
+struct alignas(16) Slots<U, false, NB> {
+  uint32_t id[NB][U];
 };
 
 // A group of LPR lanes walks a list of `nrows` rows, four columns a lane: row k's sum over its
@@ -196,19 +198,20 @@ struct alignas(16) Slots<U, false> {
 // 237 before).
 template <int LPR, int U, bool WEIGHTED, bool L2ONLY, class Bounds, class Own, class Emit>
 __device__ __forceinline__ void walk_rows(const SpmmArgs& a, const float* __restrict__ srcq,
-                                          int gl, unsigned gm, Slots<U, WEIGHTED>& slots,
-                                          int nrows, bool on, Bounds&& bounds, Own&& own,
-                                          Emit&& emit) {
+                                          int gl, unsigned gm,
+                                          Slots<U, WEIGHTED, L2ONLY ? 1 : 2>& slots, int nrows,
+                                          bool on, Bounds&& bounds, Own&& own, Emit&& emit) {
   constexpr int E = (U + LPR - 1) / LPR;  // ids a lane fetches
   constexpr bool TOGETHER = LPR < 32;
+  constexpr int NB = L2ONLY ? 1 : 2;
   const uint32_t ld = (uint32_t)a.ld;
-  auto put = [&](const uint32_t(&c)[E], const float(&w)[E]) {
+  auto put = [&](int b, const uint32_t(&c)[E], const float(&w)[E]) {
 #pragma unroll
     for (int e = 0; e < E; ++e) {
       const int k = gl + e * LPR;
       if (U % LPR != 0 && k >= U) continue;
-      slots.id[k] = c[e];
-      if constexpr (WEIGHTED) slots.w[k] = w[e];
+      slots.id[b][k] = c[e];
+      if constexpr (WEIGHTED) slots.w[b][k] = w[e];
     }
   };
   auto fetch = [&](uint32_t u, uint32_t j, int rem, uint32_t(&c)[E], float(&w)[E]) {
@@ -229,9 +232,10 @@ __device__ __forceinline__ void walk_rows(const SpmmArgs& a, const float* __rest
   if (nrows > 1) bounds(1, nj, nrem, nu);
   uint32_t c[E];
   float w[E];
+  int b = 0;  // the set that holds this step's slots
   fetch(u, j, rem, c, w);
   __syncwarp(gm);  // the group is done with the slots of an earlier walk
-  put(c, w);
+  put(0, c, w);
   __syncwarp(gm);
   Quad pu = {0, 0}, acc = {0, 0};
   bool fresh = true;
@@ -241,13 +245,13 @@ __device__ __forceinline__ void walk_rows(const SpmmArgs& a, const float* __rest
     uint32_t bj = 0, bu = 0;
     int brem = -1;
     if (last && k + 2 < nrows) bounds(k + 2, bj, brem, bu);
-    if (fresh && k < nrows) pu = own(u);
+    if (fresh && (!TOGETHER || k < nrows)) pu = own(u);
     auto step = [&](auto count) {
       constexpr int N = decltype(count)::value;
       Quad v[N];
 #pragma unroll
       for (int t = 0; t < N; t += 4) {
-        const uint4 id = *reinterpret_cast<const uint4*>(&slots.id[t]);
+        const uint4 id = *reinterpret_cast<const uint4*>(&slots.id[b][t]);
         const uint32_t ids[4] = {id.x, id.y, id.z, id.w};
 #pragma unroll
         for (int r = 0; r < 4; ++r)
@@ -259,7 +263,7 @@ __device__ __forceinline__ void walk_rows(const SpmmArgs& a, const float* __rest
 #pragma unroll
       for (int t = 0; t < N; t += 4) {
         float4 wq = make_float4(1.f, 1.f, 1.f, 1.f);
-        if constexpr (WEIGHTED) wq = *reinterpret_cast<const float4*>(&slots.w[t]);
+        if constexpr (WEIGHTED) wq = *reinterpret_cast<const float4*>(&slots.w[b][t]);
         const float ws[4] = {wq.x, wq.y, wq.z, wq.w};
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
@@ -281,10 +285,11 @@ __device__ __forceinline__ void walk_rows(const SpmmArgs& a, const float* __rest
       else if (U > 8 && most <= 8) step(ic<8>{});
       else step(ic<U>{});
     }
-    __syncwarp(TOGETHER ? 0xffffffffu : gm);  // the group is done with this step's slots
-    put(c, w);
+    if constexpr (NB == 1) __syncwarp(TOGETHER ? 0xffffffffu : gm);
+    b = NB - 1 - b;
+    put(b, c, w);  // with two sets: last read one step ago, before that step's barrier
     if (last) {
-      if (rem >= 0) emit(k, u, pu, rem > 0 ? acc : Quad{0, 0});
+      if (rem >= 0) emit(k, u, pu, TOGETHER && rem == 0 ? Quad{0, 0} : acc);
       acc = Quad{0, 0};
       ++k;
       u = nu;
@@ -486,7 +491,7 @@ template <int LPR, int VPL, bool WEIGHTED, class Own, class Emit>
 __device__ __forceinline__ void block_apply(const SpmmArgs& a, const float* src, int64_t r0,
                                             int64_t rstep, int nrows, const int* hv, int nh,
                                             int hrows, float* comb,
-                                            Slots<RUB<LPR>, WEIGHTED>& slots, int gl, int gi,
+                                            Slots<RUB<LPR>, WEIGHTED, 1>& slots, int gl, int gi,
                                             unsigned gm, unsigned on, Own&& own, Emit&& emit) {
   constexpr int GPB = PT / LPR;
   const int nvec = a.ld >> 2;
@@ -650,7 +655,7 @@ __global__ void __launch_bounds__(PT, 1) k_cg_resident(ResArgs ra) {
   __shared__ int s_iters[MAXC], s_conv[MAXC];
   __shared__ int s_nh, s_wcnt[PWARPS];
   __shared__ unsigned s_most;
-  __shared__ Slots<RUB<LPR>, WEIGHTED> slots[VPL == 1 ? GPB : 1];  // the wide rows have none
+  __shared__ Slots<RUB<LPR>, WEIGHTED, 1> slots[VPL == 1 ? GPB : 1];  // the wide rows have none
 
   // ---- which rows the block gathers in A: its own, or dealt ones where the own ranges are so
   // uneven that the largest would cost more than 4 us an iteration over the mean.  A gathered
