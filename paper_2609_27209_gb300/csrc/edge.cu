@@ -305,12 +305,14 @@ __global__ void __launch_bounds__(T)
 struct Factor {
   float a, b, c, back;
   __device__ explicit Factor(double f) {
-    const int k = f > 0.0 ? ilogb(f) : 0;
-    const double s = ldexp(f, -k);
-    a = (float)s;
-    b = (float)(s - (double)a);
-    c = (float)(s - (double)a - (double)b);
-    back = ldexpf(1.f, k);
+    // 24, 24 and 5 bits of the significand, without float64 arithmetic
+    const unsigned long long bits = (unsigned long long)__double_as_longlong(f);
+    const int k = (int)(bits >> 52) - 1023;  // f is zero or at least 2^-126
+    const unsigned long long m = f > 0.0 ? (bits & ((1ull << 52) - 1)) | 1ull << 52 : 0;
+    a = (float)(unsigned)(m >> 29) * 0x1p-23f;
+    b = (float)(unsigned)((m >> 5) & 0xffffffu) * 0x1p-47f;
+    c = (float)(unsigned)(m & 31u) * 0x1p-52f;
+    back = f > 0.0 ? __int_as_float((k + 127) << 23) : 0.f;
   }
   __device__ __forceinline__ float times(float w) const {
     const float p = __fmul_rn(w, a), pe = __fmaf_rn(w, a, -p);
