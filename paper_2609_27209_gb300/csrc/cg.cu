@@ -1321,15 +1321,19 @@ SolverPlans solver_plans(const erc_graph* g, int ld, bool pc) {
   return p;
 }
 
-// Where both single-launch solvers fit, the cheaper per iteration by a model fitted to GB300
-// timings: the resident gather costs ~2.4 ns per 128-byte neighbour line per SM plus ~18 us of
-// synchronisation and vector work; the cluster gather ~2.6 ns per neighbour per block (one
-// request per column group) plus ~10 us.  Small graphs favour the cluster solver.
+// Where both single-launch solvers fit, the cheaper per iteration by a model of their times in us,
+// fitted to uniform random graphs of 1,000 to 20,000 nodes, 3 to 12 edges a node and 16 to 256
+// columns.  Resident: 16 of synchronisation (6 more from 129 columns on, whose reductions take twice
+// the trips) and 3.2 ns a gathered 128-byte line of an SM (such graphs wait for latency; where L2
+// bounds the gathers a line costs about 1 ns).  Cluster: 7.3, 12 ns a row of a block and 1.65 ns a
+// gathered 64-byte line of it; a cluster of S blocks solves 16 columns, side by side with the
+// others.  Of 66 graphs none takes a solver more than 3% slower; with the former constants (2.4 ns a
+// line for the resident solver, from before its row walk) 5 did, by up to 38%.
 bool prefer_cluster(const erc_graph* g, int ld, const ClusterPlan& cp) {
-  const double nnz = 2.0 * (double)g->m;
+  const double nnz = 2.0 * (double)g->m, n = g->n;
   const double lines = std::max(1.0, ld / 32.0);
-  const double t_res = 18.0 + nnz * lines * 2.4e-3 / sm_count();
-  const double t_cl = 10.0 + nnz / cp.S * 2.6e-3;
+  const double t_res = 16.0 + (ld > 128 ? 6.0 : 0.0) + nnz * lines * 3.2e-3 / sm_count();
+  const double t_cl = 7.3 + (n * 12e-3 + nnz * 1.65e-3) / cp.S;
   return t_cl < t_res;
 }
 
