@@ -4,10 +4,10 @@
 // lays the canonical pairs out in lexicographic order with duplicates adjacent and in input order,
 // and one pass merges them into the numbered edge list (eu, ev, ew).  In the symmetric CSR a row's
 // smaller neighbours come first: the upper slots (row u, column v > u) are the edge list itself,
-// and the lower slots (row v, column u < v) are the edges in the order of (v, u), which a stable sort
-// of the edge list by v gives.  With U[r] and L[r] the numbers of upper and lower slots in the rows
-// before r, row_ptr[r] = U[r] + L[r]; the i-th lower slot of the whole matrix sits at U[v] + i and
-// edge e's upper slot at e + L[u + 1].
+// and the lower slots (row v, column u < v) are the edges in the order of (v, u), which a stable
+// sort of the edge list by v gives.  With U[r] and L[r] the numbers of upper and lower slots in the
+// rows before r, row_ptr[r] = U[r] + L[r]; the i-th lower slot of the whole matrix sits at U[v] + i
+// and edge e's upper slot at e + L[u + 1].
 //
 // Sorting one key an edge (and then the edges by half a key) moves less than half the bytes of
 // sorting both directions by whole keys, and every edge id is known where its slot is written: no
@@ -213,12 +213,13 @@ __global__ void __launch_bounds__(BT, MERGE_BLOCKS)
   counts_flush(h, counts, vpasses);
 }
 
-// The starts of the rows without slots in a list of m slots sorted by row: the first slot of a later
-// row, by binary search, a thread a row.  The searches of neighbouring rows take the same steps, so a
-// warp's loads are one line each and mostly in L1; a serial fill by the thread of the next slot's row
-// lasts as long as the longest run of such rows.  1M users with the smaller ids, 0.1M items, 3M edges:
-// a build of 0.73 ms (4.06 with the serial fill, 3.3 of them in one thread); 10M nodes, 0.1M edges:
-// 1.11 ms (1.93); 2.45M nodes, 64.3M edges, few such rows: 9.1 ms either way.
+// The starts of the rows without slots in a list of m slots sorted by row: the first slot of a
+// later row, by binary search, a thread a row.  The searches of neighbouring rows take the same
+// steps, so a warp's loads are one line each and mostly in L1; a serial fill by the thread of the
+// next slot's row lasts as long as the longest run of such rows.  1M users with the smaller ids,
+// 0.1M items, 3M edges: a build of 0.73 ms (4.06 with the serial fill, 3.3 of them in one thread);
+// 10M nodes, 0.1M edges: 1.11 ms (1.93); 2.45M nodes, 64.3M edges, few such rows: 9.1 ms either
+// way.
 struct RowOfEdge {
   const int32_t* eu;
   __device__ int32_t operator()(uint32_t i) const { return __ldg(eu + i); }
@@ -287,10 +288,10 @@ __global__ void __launch_bounds__(BT)
 }
 
 // A running sum in three float32 words, each addition's error carried to the next word exactly: at
-// least 70 bits, where float64 has 53.  GB300 adds float64 at a sixty-fourth of the float32 rate, and
-// the conversions run there too; three words take 13 float32 operations an addend.  The addends are
-// positive: once the sum passes the largest float the first word stays infinite, and so is the sum
-// (the other words then hold differences of infinities).
+// least 70 bits, where float64 has 53.  GB300 adds float64 at a sixty-fourth of the float32 rate,
+// and the conversions run there too; three words take 13 float32 operations an addend.  The addends
+// are positive: once the sum passes the largest float the first word stays infinite, and so is the
+// sum (the other words then hold differences of infinities).
 struct Sum3 {
   float a = 0.f, b = 0.f, c = 0.f;
   __device__ __forceinline__ void add(float x) {
@@ -305,10 +306,10 @@ struct Sum3 {
   }
 };
 
-// A row's weights summed to at least float64's precision, rounded once.  Eight lanes a row; a warp's
-// rows of more than 256 neighbours are taken by the whole warp, one after another, so that a hub
-// does not hold up its warp at eight lanes.  2.45M nodes, 64.3M edges: 367 us; 862 us with float64
-// sums, 5.4 ms with one thread a row.
+// A row's weights summed to at least float64's precision, rounded once.  Eight lanes a row; a
+// warp's rows of more than 256 neighbours are taken by the whole warp, one after another, so that a
+// hub does not hold up its warp at eight lanes.  2.45M nodes, 64.3M edges: 367 us; 862 us with
+// float64 sums, 5.4 ms with one thread a row.
 constexpr int DL = 8;
 __global__ void __launch_bounds__(BT)
     k_degree(const int64_t* __restrict__ row_ptr, const float* __restrict__ val, int32_t n,

@@ -90,7 +90,8 @@ __global__ void __launch_bounds__(T, 2) k_spmm(const __grid_constant__ SpmmArgs 
   const int nvec = a.ld >> 2;
   const unsigned gm = group_mask<LPR>();
   const int64_t nheavy = a.nheavy ? *a.nheavy : 0;
-  const int hmine = nheavy > blockIdx.x ? (int)((nheavy - blockIdx.x + gridDim.x - 1) / gridDim.x) : 0;
+  const int hmine =
+      nheavy > blockIdx.x ? (int)((nheavy - blockIdx.x + gridDim.x - 1) / gridDim.x) : 0;
   const uint32_t u0 = blockIdx.x * GPB + gi, ustep = gridDim.x * GPB;
   const int mine = (uint32_t)a.n > u0 ? (int)(((uint32_t)a.n - u0 + ustep - 1) / ustep) : 0;
   for (int q0 = 0; q0 < nvec; q0 += LPR) {
@@ -391,9 +392,9 @@ __global__ void __launch_bounds__(T) k_update_fused(VecArgs a) {
   const bool any_p = act.x | act.y | act.z | act.w;
   const bool any_x = al.x != 0.f || al.y != 0.f || al.z != 0.f || al.w != 0.f;
   if (!any_x && !any_p) return;
-  // The rows backwards: the r rows that the first part wrote last are still in L2 (none of the first
-  // rows are, once a block of vectors exceeds it).  x is touched here alone, so it streams past.
-  // 169k nodes x 256 columns: a solve 126.0 -> 124.7 ms.
+  // The rows backwards: the r rows that the first part wrote last are still in L2 (none of the
+  // first rows are, once a block of vectors exceeds it).  x is touched here alone, so it streams
+  // past.  169k nodes x 256 columns: a solve 126.0 -> 124.7 ms.
   const int64_t chunks = (a.n - row0 + UPD * rstep - 1) / (UPD * rstep);
   for (int64_t c = chunks - 1; c >= 0; --c) {
     const int64_t rowb = row0 + c * UPD * rstep;
@@ -440,13 +441,14 @@ __global__ void __launch_bounds__(T) k_update_fused(VecArgs a) {
 // a thread-block cluster of CS blocks owns a group of 16 columns for every row and runs the whole
 // solve of its group; clusters never wait on one another.  Block k of a cluster owns the rows
 // [b_k, b_k+1) (equal shares of the neighbour lists, at most rbmax rows): their r and Ap live in
-// its shared memory, and with PX x and a copy of p too; p is in global memory (it is gathered by the
-// cluster's other blocks, from L2), and so is x without PX.  Four lanes take one light row, a float4 of the group's columns each, so a neighbour costs
-// one 64-byte line; the next row's bounds and column indices are fetched while the current row's
-// neighbours are in flight.  Rows heavier than H are split over the whole block.  Per-column dot
-// products are combined in a fixed order: within a block by warp shuffles and shared memory,
-// across the cluster by every block reading every block's partial through distributed shared
-// memory, so all blocks of a cluster derive the same alpha, beta and stop decisions.
+// its shared memory, and with PX x and a copy of p too; p is in global memory (it is gathered by
+// the cluster's other blocks, from L2), and so is x without PX.  Four lanes take one light row, a
+// float4 of the group's columns each, so a neighbour costs one 64-byte line; the next row's bounds
+// and column indices are fetched while the current row's neighbours are in flight.  Rows heavier
+// than H are split over the whole block.  Per-column dot products are combined in a fixed order:
+// within a block by warp shuffles and shared memory, across the cluster by every block reading
+// every block's partial through distributed shared memory, so all blocks of a cluster derive the
+// same alpha, beta and stop decisions.
 // Per iteration: A (Ap, p.Ap) | B (x, r, r.r) | C (p), each closed by a hardware cluster barrier.
 constexpr int CT = 384;
 constexpr int CWARPS = CT / 32;
@@ -1268,8 +1270,8 @@ bool cluster_plan_for(const erc_graph* g, int ld, bool px, ClusterPlan* pl) {
 }
 
 // The largest cluster decides (it is what the solve's time depends on); where the same one and the
-// same row split hold p and x of a block's rows in shared memory too, they stay there: the vector phases then wait on no load
-// (2,000 nodes, 64 columns: 282 us a solve, 300 us with both in L2).
+// same row split hold p and x of a block's rows in shared memory too, they stay there: the vector
+// phases then wait on no load (2,000 nodes, 64 columns: 282 us a solve, 300 us with both in L2).
 bool cluster_plan(const erc_graph* g, int ld, ClusterPlan* pl) {
   ClusterPlan px;
   if (!cluster_plan_for(g, ld, false, pl)) return false;
@@ -1323,12 +1325,12 @@ SolverPlans solver_plans(const erc_graph* g, int ld, bool pc) {
 
 // Where both single-launch solvers fit, the cheaper per iteration by a model of their times in us,
 // fitted to uniform random graphs of 1,000 to 20,000 nodes, 3 to 12 edges a node and 16 to 256
-// columns.  Resident: 16 of synchronisation (6 more from 129 columns on, whose reductions take twice
-// the trips) and 3.2 ns a gathered 128-byte line of an SM (such graphs wait for latency; where L2
-// bounds the gathers a line costs about 1 ns).  Cluster: 7.3, 12 ns a row of a block and 1.65 ns a
-// gathered 64-byte line of it; a cluster of S blocks solves 16 columns, side by side with the
-// others.  Of 66 graphs none takes a solver more than 3% slower; with the former constants (2.4 ns a
-// line for the resident solver, from before its row walk) 5 did, by up to 38%.
+// columns.  Resident: 16 of synchronisation (6 more from 129 columns on, whose reductions take
+// twice the trips) and 3.2 ns a gathered 128-byte line of an SM (such graphs wait for latency;
+// where L2 bounds the gathers a line costs about 1 ns).  Cluster: 7.3, 12 ns a row of a block and
+// 1.65 ns a gathered 64-byte line of it; a cluster of S blocks solves 16 columns, side by side with
+// the others.  Of 66 graphs none takes a solver more than 3% slower; with the former constants (2.4
+// ns a line for the resident solver, from before its row walk) 5 did, by up to 38%.
 bool prefer_cluster(const erc_graph* g, int ld, const ClusterPlan& cp) {
   const double nnz = 2.0 * (double)g->m, n = g->n;
   const double lines = std::max(1.0, ld / 32.0);

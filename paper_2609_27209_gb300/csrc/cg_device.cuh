@@ -142,8 +142,8 @@ __device__ __forceinline__ Quad ld_quad(const float* p) {
   return quad(L2ONLY ? __ldcg(reinterpret_cast<const float4*>(p)) : ld_f4(p));
 }
 
-// Four columns at p, past L1, where `on`, else v.  A predicated load: a branch would make the lanes of
-// its two sides wait one after the other.
+// Four columns at p, past L1, where `on`, else v.  A predicated load: a branch would make the lanes
+// of its two sides wait one after the other.
 __device__ __forceinline__ Quad ldcg_quad_if(bool on, const float* p, Quad v) {
   asm volatile(
       "{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %3, 0;\n\t"
@@ -161,10 +161,10 @@ __device__ __forceinline__ float4 ldcg_f4_if(bool on, const float* p, float4 v) 
   return v;
 }
 
-// The neighbour ids (and weights) of a group's step, in shared memory: the step reads four at a time,
-// where lanes that passed each other the ids would take a shuffle for every slot.  With NB = 2 the
-// next step's are put beside this step's; with one set, in the resident solver, whose rows compete for
-// the memory, they wait until the group is done with them.
+// The neighbour ids (and weights) of a group's step, in shared memory: the step reads four at a
+// time, where lanes that passed each other the ids would take a shuffle for every slot.  With
+// NB = 2 the next step's are put beside this step's; with one set, in the resident solver, whose
+// rows compete for the memory, they wait until the group is done with them.
 template <int U, bool WEIGHTED, int NB>
 struct alignas(16) Slots {
   uint32_t id[NB][U];
@@ -186,16 +186,16 @@ struct alignas(16) Slots<U, false, NB> {
 // enough of them are in flight: what bounds a walk is the latency of the chain row bounds ->
 // neighbour ids -> neighbour rows.  So the chain is taken apart: a step gathers up to U rows at
 // once, and while they are on their way the next step's ids are loaded, which at a row's end are
-// the next row's first, and the bounds of the row after that.  The short last step of a row takes 4,
-// 8 or U slots; those past the end hold the row itself.  Through L1 they are loaded, from a cached line,
-// and add exactly zero (128 columns, 150k nodes, 1.5M edges: 130 us, 139 with the loads predicated
-// off).  Past L1 each would be a request to L2, so they are predicated off, and p_u stands for them
-// (20,000 nodes, 160,000 edges, 32 columns: 477 us a solve, 544 with them).
+// the next row's first, and the bounds of the row after that.  The short last step of a row takes
+// 4, 8 or U slots; those past the end hold the row itself.  Through L1 they are loaded, from a
+// cached line, and add exactly zero (128 columns, 150k nodes, 1.5M edges: 130 us, 139 with the
+// loads predicated off).  Past L1 each would be a request to L2, so they are predicated off, and
+// p_u stands for them (20,000 nodes, 160,000 edges, 32 columns: 477 us a solve, 544 with them).
 //
 // The groups of a warp take their steps together, with the longest one's count: left to themselves
-// they drift apart, and a warp then issues, and waits for, each group's gathers in turn (1M nodes, 8M
-// edges of a power law, 32 columns: 383 us an application, 508 before; 1M nodes, 3M edges: 178 us,
-// 237 before).
+// they drift apart, and a warp then issues, and waits for, each group's gathers in turn (1M nodes,
+// 8M edges of a power law, 32 columns: 383 us an application, 508 before; 1M nodes, 3M edges:
+// 178 us, 237 before).
 template <int LPR, int U, bool WEIGHTED, bool L2ONLY, class Bounds, class Own, class Emit>
 __device__ __forceinline__ void walk_rows(const SpmmArgs& a, const float* __restrict__ srcq,
                                           int gl, unsigned gm,
@@ -432,14 +432,15 @@ __host__ __device__ constexpr size_t resident_shared_floats(int hrows, int vpl) 
   return 4 * (size_t)PT * (size_t)(hrows * vpl);
 }
 
-// acc[v] += w (p_u - p_v) over the CSR slots [j, j + len) of row u, for the lane's VPL quads of every
-// neighbour at once: rows of more than 128 columns.  The ids pass by shuffles, and 8 / VPL neighbours
-// are in flight.  A walk for each quad passes over the row bounds and ids twice and waits twice
-// (10,000 nodes, 256 columns: 60,000 edges 976 us a solve, 881 with both quads at once, 875 before
-// the walk; 120,000 edges 1,130, 901 and 890).
+// acc[v] += w (p_u - p_v) over the CSR slots [j, j + len) of row u, for the lane's VPL quads of
+// every neighbour at once: rows of more than 128 columns.  The ids pass by shuffles, and 8 / VPL
+// neighbours are in flight.  A walk for each quad passes over the row bounds and ids twice and
+// waits twice (10,000 nodes, 256 columns: 60,000 edges 976 us a solve, 881 with both quads at once,
+// 875 before the walk; 120,000 edges 1,130, 901 and 890).
 template <int LPR, int VPL, bool WEIGHTED>
-__device__ __forceinline__ void gather_wide(const SpmmArgs& a, const float* __restrict__ src, int gl,
-                                            unsigned gm, int nvec, unsigned on, uint32_t j, int len,
+__device__ __forceinline__ void gather_wide(const SpmmArgs& a, const float* __restrict__ src,
+                                            int gl, unsigned gm, int nvec, unsigned on,
+                                            uint32_t j, int len,
                                             const float4 (&pu)[VPL], float4 (&acc)[VPL]) {
   constexpr int U = 8 / VPL;
   for (int jb = 0; jb < len; jb += LPR) {
@@ -659,8 +660,9 @@ __global__ void __launch_bounds__(PT, 1) k_cg_resident(ResArgs ra) {
 
   // ---- which rows the block gathers in A: its own, or dealt ones where the own ranges are so
   // uneven that the largest would cost more than 4 us an iteration over the mean.  A gathered
-  // 128-byte line costs about 1 ns of an SM (the gathers run at 13 to 20 TB/s over 152 SMs): 4,000
-  // lines, where handing Ap over through L2 costs under a microsecond.  Every block finds the same.
+  // 128-byte line costs about 1 ns of an SM where L2 bounds the gathers (13 to 20 TB/s over 152
+  // SMs): 4,000 lines, where handing Ap over through L2 costs under a microsecond.  Every block
+  // finds the same.
   if (threadIdx.x == 0) {
     s_nh = 0;
     s_most = 0;

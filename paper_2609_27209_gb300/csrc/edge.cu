@@ -25,13 +25,13 @@ __device__ __forceinline__ float4 ld_f4(const float* p) {
 // its bits do not change.  The group owns each R_e it touches: no atomics.
 // The rows X_v are random reads, bound by HBM where X exceeds L2 (7.4 TB/s for such reads).  Four
 // edges a step and four blocks an SM: 2.45M nodes, 64.3M edges, 128 columns, distances to
-// probabilities: 7.73 -> 6.81 ms (eight edges 7.46 with three blocks and 8.01 with four; five blocks
-// 7.96), with both rows loaded for every edge before.
-// Wider rows, with the blocks an SM that their registers allow; from 257 columns on every lane loads the
+// probabilities: 7.73 -> 6.81 ms (eight edges 7.46 with three blocks and 8.01 with four; five
+// blocks 7.96), with both rows loaded for every edge before.
+// Wider rows: the blocks an SM that their registers allow; from 257 columns on every lane loads the
 // ids itself, because a group is a warp there and the shuffles are on the path to the first row.
 // 1M nodes, 8M edges, 192 columns: 0.95 ms (1.04 with both rows for every edge, 1.16 with three
-// blocks); 20,000 nodes, 200,000 edges, 384 columns: 43.4 us (43.5, and 49.1 with one edge a step in two
-// blocks and ids by shuffles).
+// blocks); 20,000 nodes, 200,000 edges, 384 columns: 43.4 us (43.5, and 49.1 with one edge a step
+// in two blocks and ids by shuffles).
 template <int LPR, int VPL>
 __global__ void __launch_bounds__(T, VPL <= 2 ? 4 : VPL == 4 ? 3 : 2)
     k_edge_resistance(const int32_t* __restrict__ eu, const int32_t* __restrict__ ev, int64_t m,
@@ -72,7 +72,8 @@ __global__ void __launch_bounds__(T, VPL <= 2 ? 4 : VPL == 4 ? 3 : 2)
 #pragma unroll
         for (int t = 0; t < VPL; ++t) {
           const int q = gl + LPR * t;
-          xv[k][t] = q < nvec ? ld_f4(X + (size_t)v[k] * ld + 4 * q) : make_float4(0.f, 0.f, 0.f, 0.f);
+          xv[k][t] = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (q < nvec) xv[k][t] = ld_f4(X + (size_t)v[k] * ld + 4 * q);
         }
 #pragma unroll
       for (int k = 0; k < EB; ++k)
@@ -80,7 +81,8 @@ __global__ void __launch_bounds__(T, VPL <= 2 ? 4 : VPL == 4 ? 3 : 2)
         for (int t = 0; t < VPL; ++t) {
           const int q = gl + LPR * t;
           xu[k][t] = make_float4(0.f, 0.f, 0.f, 0.f);
-          if (q < nvec && (k == 0 || u[k] != u[k - 1])) xu[k][t] = ld_f4(X + (size_t)u[k] * ld + 4 * q);
+          if (q < nvec && (k == 0 || u[k] != u[k - 1]))
+            xu[k][t] = ld_f4(X + (size_t)u[k] * ld + 4 * q);
         }
 #pragma unroll
       for (int k = 0; k < EB; ++k) {
@@ -299,9 +301,9 @@ __global__ void __launch_bounds__(T)
   }
 }
 
-// A float64 factor f in [0, 1] as three float32 words (all of its 53 bits, scaled to [1, 2] so that no
-// part of a product underflows), and w f to at least 68 bits, rounded once.  The float64 product is
-// rounded to 53 bits first, and GB300 runs it at a sixty-fourth of the float32 rate.
+// A float64 factor f in [0, 1] as three float32 words (all of its 53 bits, scaled to [1, 2] so that
+// no part of a product underflows), and w f to at least 68 bits, rounded once.  The float64 product
+// is rounded to 53 bits first, and GB300 runs it at a sixty-fourth of the float32 rate.
 struct Factor {
   float a, b, c, back;
   __device__ explicit Factor(double f) {

@@ -375,8 +375,8 @@ __device__ __forceinline__ void colsum_rows(const float2* part, int G, int ld, f
 }
 
 // colsum_rows for float partials (part: [G][ld] floats, ld a multiple of 4, ld <= 2 blockDim.x):
-// four columns per load, float-pair sums in a fixed order; tmp holds 2 * blockDim.x entries.  For partials that are sums of squares, whose
-// rounding to float costs at most 2^-24 of the total.
+// four columns per load, float-pair sums in a fixed order; tmp holds 2 * blockDim.x entries.  For
+// partials that are sums of squares, whose rounding to float costs at most 2^-24 of the total.
 __device__ __forceinline__ void colsum_rows_f(const float* part, int G, int ld, float2* res,
                                               float2* tmp) {
   const int bd = blockDim.x;
@@ -476,10 +476,10 @@ erc_status check_graph(const erc_graph* g);
 constexpr unsigned LOOKBACK_SPINS = 1u << 22;  // polls of a predecessor tile before giving up
 // Passes of a stable LSD radix sort of (key, value) pairs by 8-bit digits.  The caller zeroes the
 // temporary storage once (radix_sort_begin) and numbers its passes 0, 1, ..., also across several
-// sorts that share it; n_max (at most 2^30) bounds every one of them.  A pass sorts by key bits [shift, shift +
-// 8) the first min(n_max, *n) pairs (all n_max when n, a device pointer, is null); vals may be null.
-// counts[RS_RADIX] (device) holds how many of those keys have each digit.   `abort`: the call's
-// abort word; once it is set no further pass runs and the result is undefined.
+// sorts that share it; n_max (at most 2^30) bounds every one of them.  A pass sorts by key bits
+// [shift, shift + 8) the first min(n_max, *n) pairs (all n_max when n, a device pointer, is null);
+// vals may be null.  counts[RS_RADIX] (device) holds how many of those keys have each digit.
+// `abort`: the call's abort word; once it is set no further pass runs and the result is undefined.
 constexpr int RS_BITS = 8;
 constexpr int RS_MAX_PASSES = 16;
 size_t radix_sort_temp_bytes(int64_t n_max);

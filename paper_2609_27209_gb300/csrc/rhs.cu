@@ -14,7 +14,7 @@ namespace {
 // leaves them in shared memory with the slot's coefficient; the slots are then applied in CSR
 // order, each lane reading the one word that holds its four columns' signs.  The orientation sigma
 // goes into the words (all signs of a slot flipped), and a sign is applied by moving its bit to the
-// coefficient's sign bit, two columns an addition.
+// coefficient's sign bit.
 //
 // What bounds it is instruction issue: each of the 2m slots costs a lane two shared loads and a
 // dozen operations (passing the words by shuffles, four a slot and the selection of one of them,
@@ -23,7 +23,8 @@ template <int LPR, int VPL, bool WEIGHTED>
 __global__ void __launch_bounds__(256)
     k_jl_rhs(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
              const float* __restrict__ val, const int32_t* __restrict__ csr_eid, int32_t n,
-             uint2 key, float inv_sqrt_k, int32_t c0, int32_t kc, int32_t ld, float* __restrict__ Y) {
+             uint2 key, float inv_sqrt_k, int32_t c0, int32_t kc, int32_t ld,
+             float* __restrict__ Y) {
   constexpr int NB = (4 * LPR * VPL + 127) / 128 + 1;  // 128-column Philox blocks a group can span
   constexpr int GPB = 256 / LPR;
   // a slot's words; groups are padded apart so that they meet in different banks
@@ -61,7 +62,8 @@ __global__ void __launch_bounds__(256)
     fetch(j0 + gl);
     for (int64_t jb = j0; jb < j1; jb += LPR) {
       if (jb + gl < j1) {
-        const uint32_t flip = other < u ? ~0u : 0u;  // u is the larger endpoint: row e is e_nb - e_u
+        // u is the larger endpoint: row e is e_nb - e_u
+        const uint32_t flip = other < u ? ~0u : 0u;
 #pragma unroll
         for (int b = 0; b < NB; ++b) {
           if (b >= nb) break;

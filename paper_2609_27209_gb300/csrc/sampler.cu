@@ -25,7 +25,7 @@ namespace {
 constexpr int ST = 256;
 constexpr int SWARPS = ST / 32;
 // Entries per thread of a scan or compaction tile: 32 from SLARGE entries on, so that the look-back
-// over the tiles in flight stays short, 8 below, so that a small graph's passes spread over the SMs.
+// over the tiles in flight stays short, 8 below, so that a small graph's passes spread over SMs.
 constexpr int SIPT_LARGE = 32, SIPT_SMALL = 8;
 constexpr int64_t SLARGE = 1 << 20;
 constexpr int SMID = 64;
@@ -40,9 +40,9 @@ struct SamplePlan {
   size_t words;
   unsigned* err;  // [0] the abort word; [1..3] the passes' tickets
 };
-// Bits of the abort word.  Once one is set the passes that follow write nothing: a call that reports
-// an error leaves its outputs alone.  (A word of its own for each reason, read by every block of the
-// compactions, took 3% to 12% of a call.)
+// Bits of the abort word.  Once one is set the passes that follow write nothing: a call that
+// reports an error leaves its outputs alone.  (A word of its own for each reason, read by every
+// block of the compactions, took 3% to 12% of a call.)
 constexpr unsigned WAIT_RAN_OUT = 1, BAD_PROB = 2, NO_WEIGHT = 4;  // tile_prefix sets the first
 
 inline int64_t stile(int64_t count) { return ST * (count < SLARGE ? SIPT_SMALL : SIPT_LARGE); }
@@ -63,8 +63,8 @@ inline int64_t mark_bytes_max(int64_t n) {
   return std::max(n, std::min(MARK_COPIES * n, MARK_BYTES));
 }
 
-// The plan of every call on a graph of n nodes and m edges, drawn by node or by edge.  No array shrinks
-// as n or m grows, so a workspace serves every graph up to the sizes it was reported for.
+// The plan of every call on a graph of n nodes and m edges, drawn by node or by edge.  No array
+// shrinks as n or m grows, so a workspace serves every graph up to the sizes it was reported for.
 void plan_sample(Arena& a, SamplePlan& p, int32_t n, int64_t m) {
   const int64_t count = std::max<int64_t>(n, m);  // entries drawn from, at most
   p.E = a.take<int64_t>(count);
@@ -105,7 +105,8 @@ __device__ __forceinline__ int64_t claim_tile(unsigned* ticket, const unsigned* 
 }
 
 // E, Emid and T of the weights.  A warp takes 32 SIPT consecutive entries, a lane four neighbouring
-// ones of each 128, so that a scan over the lanes serves 128 entries; `vec`: prob is 16-byte aligned.
+// ones of each 128, so that a scan over the lanes serves 128 entries; `vec`: prob is 16-byte
+// aligned.
 template <int SIPT>
 __global__ void __launch_bounds__(ST)
     k_weight_scan(const float* __restrict__ prob, int64_t count, bool vec, int64_t* __restrict__ E,
@@ -190,17 +191,18 @@ __global__ void __launch_bounds__(ST)
   }
 }
 
-// draw k: the largest i with E_i <= floor(x_k T / 2^64), found in the scan's tiles (their final status
-// words hold the sums with each tile: a few KB that stay in L1), then in Emid (L2), then among the
-// SMID entries of E it leads to: a plain binary search over E misses L2 about eight times a draw
-// on 64M entries.  Marks node i, or edge i's endpoints and, where emark is not null, the edge.
-// Stores to one line queue up in L2, and a power-law graph's draws keep hitting the lines of its
-// hubs: the blocks spread them over `copies` arrays of marks, which the compaction joins.  (Testing a
-// mark before storing it queues the test behind the stores: 276 us against 31 for 129k draws
-// over 6,821 nodes.)
+// draw k: the largest i with E_i <= floor(x_k T / 2^64), found in the scan's tiles (their final
+// status words hold the sums with each tile: 8 bytes a tile, 63 KB for 64M entries), then in Emid
+// (L2), then among the SMID entries of E it leads to: a plain binary search over E misses L2 about
+// eight times a draw on 64M entries.  Marks node i, or edge i's endpoints and, where emark is not
+// null, the edge.  Stores to one line queue up in L2, and a power-law graph's draws keep hitting
+// the lines of its hubs: the blocks spread them over `copies` arrays of marks, which the compaction
+// joins.  (Testing a mark before storing it queues the test behind the stores: 276 us against 31
+// for 129k draws over 6,821 nodes.)
 __global__ void __launch_bounds__(ST)
-    k_draw(const int64_t* __restrict__ E, const int64_t* __restrict__ Emid, int64_t count, int64_t tile,
-           const unsigned long long* __restrict__ status, const int64_t* __restrict__ tot,
+    k_draw(const int64_t* __restrict__ E, const int64_t* __restrict__ Emid, int64_t count,
+           int64_t tile, const unsigned long long* __restrict__ status,
+           const int64_t* __restrict__ tot,
            int64_t budget, uint2 key, int64_t first, uint32_t stream,
            const int32_t* __restrict__ eu, const int32_t* __restrict__ ev,
            uint8_t* __restrict__ nmark, int32_t n, int copies, uint8_t* __restrict__ emark,
@@ -411,8 +413,9 @@ extern "C" erc_status erc_sample_subgraph(const erc_graph* g, int32_t kind, cons
   const int copies = mark_copies(g->n);
   ERC_CUDA(cudaMemsetAsync(p.nmark, 0, (size_t)g->n * copies, s));
   if (drawn_edges) ERC_CUDA(cudaMemsetAsync(p.emark, 0, (size_t)g->m, s));
-  // Nothing is read back before the end.  A wait that gives up within a compaction leaves its output
-  // incomplete; the prefixes are then below their true values, so every index stays in range.
+  // Nothing is read back before the end.  A wait that gives up within a compaction leaves its
+  // output incomplete; the prefixes are then below their true values, so every index stays in
+  // range.
   const unsigned limit = wait_limit(LOOKBACK_SPINS);
   const bool vec = (reinterpret_cast<uintptr_t>(prob) & 15) == 0;
   if (count < SLARGE)
@@ -434,8 +437,8 @@ extern "C" erc_status erc_sample_subgraph(const erc_graph* g, int32_t kind, cons
                   p.status_n, p.err + 2, abort, limit, s));
   if (g->m > 0) {
     if (drawn_edges)
-      ERC_TRY(compact(MarkedFlag{p.emark}, g->m, edges, (uint32_t*)nullptr, &p.totals[2], p.status_m,
-                      p.err + 3, abort, limit, s));
+      ERC_TRY(compact(MarkedFlag{p.emark}, g->m, edges, (uint32_t*)nullptr, &p.totals[2],
+                      p.status_m, p.err + 3, abort, limit, s));
     else
       ERC_TRY(compact(InducedFlag{g->eu, g->ev, p.nbits}, g->m, edges, (uint32_t*)nullptr,
                       &p.totals[2], p.status_m, p.err + 3, abort, limit, s));

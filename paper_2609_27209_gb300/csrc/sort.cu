@@ -9,28 +9,29 @@ namespace erc {
 namespace {
 
 // ------------------------------------------------------------------------------------------------
-// Stable LSD radix sort of (u64 key, u32 value) pairs, one kernel per 8-bit digit (the digit counts
-// of every pass come from the kernel that wrote the keys): a tile ranks its keys, publishes its
-// digit counts, learns the counts of the tiles before it by decoupled look-back (as tile_prefix, one
-// digit per thread) and writes its keys.  HBM would bound a pass at 0.23 ms for 65.6M pairs (12 bytes
-// read and written each); the chain of a tile's phases makes it 0.62 ms, so as many tiles as fit
-// overlap on an SM.  The tile is brought into digit order in shared memory first, so that a digit's
-// keys leave as one run (10 keys, 80 bytes on average) instead of one 8-byte and one 4-byte store
-// each (the three kernels per pass it replaces -- count, scan, scatter straight from registers --
-// took 3.8 ms for 131M pairs).
-// A block's tile is split into warp sub-tiles in warp-striped order so that (warp, step, lane)
-// order equals key order, which makes the ranks stable.
-// A status word holds count << 16 | pass << 2 | flag (1 the tile's count, 2 with all tiles before):
-// no pass needs its status cleared.  Keys and values take turns in the shared buffer.
+// Stable LSD radix sort of (u64 key, u32 value) pairs, one kernel per 8-bit digit, the method of
+// A. Adinets, D. Merrill, "Onesweep: A Faster Least Significant Digit Radix Sort for GPUs", 2022
+// (the digit counts of every pass come from the kernel that wrote the keys): a tile ranks its keys,
+// publishes its digit counts, learns the counts of the tiles before it by decoupled look-back (as
+// tile_prefix, one digit per thread) and writes its keys.  HBM would bound a pass at 0.23 ms for
+// 65.6M pairs (12 bytes read and written each); the chain of a tile's phases makes it 0.62 ms, so
+// as many tiles as fit overlap on an SM.  The tile is brought into digit order in shared memory
+// first, so that a digit's keys leave as one run (10 keys, 80 bytes on average) instead of one
+// 8-byte and one 4-byte store each (the three kernels per pass it replaces -- count, scan, scatter
+// straight from registers -- took 3.8 ms for 131M pairs).  A block's tile is split into warp
+// sub-tiles in warp-striped order so that (warp, step, lane) order equals key order, which makes
+// the ranks stable.  A status word holds count << 16 | pass << 2 | flag (1 the tile's count, 2 with
+// all tiles before): no pass needs its status cleared.  Keys and values take turns in the shared
+// buffer.
 constexpr int RS_THREADS = 256;  // one digit per thread
 constexpr int RS_WARPS = RS_THREADS / 32;
 constexpr int RS_RADIX = 1 << RS_BITS;
 static_assert(RS_RADIX == RS_THREADS, "one digit per thread");
 constexpr int LB = 8;
-// Tiles of 256 x 10 keys, which leave four blocks an SM their registers (65.6M edges: 9.3 ms a build;
-// 12 keys a thread 10.1 with spills or 10.6 with three blocks, 16 keys 10.6); below RS_SMALL keys
-// 256 x 8, so that a small graph's passes spread over more SMs (2,000-node run: 22 us less than
-// with 16).
+// Tiles of 256 x 10 keys, which leave four blocks an SM their registers (65.6M edges: 9.1 ms a
+// build; 12 keys a thread 10.1 with spills or 10.6 with three blocks, 16 keys 10.6); below RS_SMALL
+// keys 256 x 8, so that a small graph's passes spread over more SMs (2,000-node run: 22 us less
+// than with 16).
 constexpr int64_t RS_SMALL = 2 << 20;
 
 template <int IPT>
@@ -221,9 +222,9 @@ void launch_pass(const uint64_t* keys, const uint32_t* vals, uint64_t* keys_out,
 }
 }  // namespace
 
-// tmp: [tickets][status: tiles x RS_RADIX].  Just below RS_SMALL keys there are more tiles than from
-// there on (1,024 against 820); the size covers the most tiles of n keys or fewer, so that storage
-// sized for a larger input serves a smaller one.  A tile's status words start on a line.
+// tmp: [tickets][status: tiles x RS_RADIX].  Just below RS_SMALL keys there are more tiles than
+// from there on (1,024 against 820); the size covers the most tiles of n keys or fewer, so that
+// storage sized for a larger input serves a smaller one.  A tile's status words start on a line.
 constexpr size_t RS_TICKETS = 256;  // bytes
 static_assert(RS_MAX_PASSES * sizeof(unsigned) <= RS_TICKETS, "a ticket a pass");
 inline size_t sort_tmp_bytes(int64_t tiles) {
@@ -250,8 +251,8 @@ erc_status radix_sort_pass(const uint64_t* keys, const uint32_t* vals, uint64_t*
     launch_pass<8>(keys, vals, keys_out, vals_out, n_max, n, shift, pass, counts, status, ticket, s,
                    abort);
   else
-    launch_pass<10>(keys, vals, keys_out, vals_out, n_max, n, shift, pass, counts, status, ticket, s,
-                    abort);
+    launch_pass<10>(keys, vals, keys_out, vals_out, n_max, n, shift, pass, counts, status, ticket,
+                    s, abort);
   count_launches(1);
   ERC_CUDA(cudaGetLastError());
   return ERC_OK;
