@@ -66,6 +66,37 @@ void plan_cg(Arena& a, CgWork& w, int32_t n, int32_t ld) {
 }
 
 
+// the blocks' column partials (sbuf) to the scalars of the step, the caller's p.Ap or the residuals
+template <int MODE>
+__device__ __forceinline__ void finish_columns(const SpmmArgs& a, float2* sbuf) {
+  if (!grid_colreduce(a.cr, sbuf, sbuf, a.ld)) return;
+  for (int c = threadIdx.x; c < a.ld; c += blockDim.x) {
+    const double v = df_value(sbuf[c]);
+    if (MODE == MODE_STEP) {
+      float al = 0.f;
+      if (a.active[c]) {
+        const double q = a.rr[c] / v;
+        if (!(v > 0.0) || !isfinite(q)) {
+          a.active[c] = 0;
+          atomicOr(&a.flags[1], 1);
+        } else {
+          al = (float)q;
+        }
+      }
+      a.alpha[c] = al;
+    } else if (MODE == MODE_APPLY) {
+      if (c < a.kc) a.pap_out[c] = v;
+    } else {
+      if (c < a.kc) {
+        const double y2 = a.yy[c];
+        a.relres_out[c] = y2 > 0.0 ? (float)sqrt(v / y2) : 0.f;
+        a.iters_out[c] = a.iters[c];
+        if (!a.conv[c]) atomicAdd(&a.flags[2], 1);
+      }
+    }
+  }
+}
+
 // One thread group per light row; the blocks' groups split the heavy rows, HB of them between two
 // barriers, and their slices are added in group order.  Rows wider than 128 columns are taken 128
 // columns at a time, so that a walk's registers hold 16 rows in flight whatever the width.
@@ -164,32 +195,104 @@ __global__ void __launch_bounds__(T, 2) k_spmm(const __grid_constant__ SpmmArgs 
                                                   min(4 * LPR, a.ld - 4 * q0));
   }
   if (MODE == MODE_APPLY && a.pap_out == nullptr) return;
-  if (!grid_colreduce(a.cr, sbuf, sbuf, a.ld)) return;
-  for (int c = threadIdx.x; c < a.ld; c += blockDim.x) {
-    const double v = df_value(sbuf[c]);
-    if (MODE == MODE_STEP) {
-      float al = 0.f;
-      if (a.active[c]) {
-        const double q = a.rr[c] / v;
-        if (!(v > 0.0) || !isfinite(q)) {
-          a.active[c] = 0;
-          atomicOr(&a.flags[1], 1);
-        } else {
-          al = (float)q;
-        }
-      }
-      a.alpha[c] = al;
-    } else if (MODE == MODE_APPLY) {
-      if (c < a.kc) a.pap_out[c] = v;
-    } else {
-      if (c < a.kc) {
-        const double y2 = a.yy[c];
-        a.relres_out[c] = y2 > 0.0 ? (float)sqrt(v / y2) : 0.f;
-        a.iters_out[c] = a.iters[c];
-        if (!a.conv[c]) atomicAdd(&a.flags[2], 1);
-      }
+  finish_columns<MODE>(a, sbuf);
+}
+
+// The operator for rows of 385 to 512 columns of a small block: a warp takes a row's four quads a
+// lane at once, two neighbours in flight.  Four slices of k_spmm each fill their pipeline anew, and
+// such graphs have only a few rows a group to spread that over.  512 columns: 20,000 nodes, 80,000
+// edges 41 us against 49 in slices; 3,000 nodes, 30,000 edges 26 against 31.  From P = 82 MB on the
+// slices are as fast or faster (40,000 nodes, 400,000 edges 136 against 131; 80,000 nodes,
+// 800,000 edges 360 against 253), as are three slices (384 columns, 20,000 nodes: 61 against 57).
+constexpr int WIDE = 4;  // quads a lane
+inline bool spmm_wide(int64_t n, int ld) {
+  return ld > 384 && ld <= 512 && n * ld * 4 <= (int64_t(64) << 20);
+}
+
+template <bool WEIGHTED, int MODE>
+__global__ void __launch_bounds__(T, 2) k_spmm_wide(const __grid_constant__ SpmmArgs a) {
+  if (MODE == MODE_STEP && (*(volatile int*)a.flags == 0 || *(volatile int*)(a.flags + 3) != 0))
+    return;
+  constexpr int LPR = 32, GPB = T / LPR;
+  __shared__ float4 part[WIDE][T];  // a heavy row's slices, then the dot products' scratch
+  __shared__ float2 sbuf[MAX_LD];
+  const int gl = threadIdx.x & (LPR - 1), gi = threadIdx.x / LPR;
+  const int nvec = a.ld >> 2;
+  float2 dot[WIDE][4];
+#pragma unroll
+  for (int v = 0; v < WIDE; ++v)
+#pragma unroll
+    for (int t = 0; t < 4; ++t) dot[v][t] = make_float2(0.f, 0.f);
+  auto load = [&](int64_t u, float4(&pu)[WIDE], float4(&acc)[WIDE]) {
+#pragma unroll
+    for (int v = 0; v < WIDE; ++v) {
+      const int q = gl + LPR * v;
+      pu[v] = q < nvec ? ld_f4(a.P + (size_t)u * a.ld + 4 * q) : f4_zero();
+      acc[v] = f4_zero();
     }
+  };
+  // L_eps p_u as in k_spmm
+  auto finish = [&](int64_t u, const float4(&pu)[WIDE], const float4(&acc)[WIDE]) {
+#pragma unroll
+    for (int v = 0; v < WIDE; ++v) {
+      const int q = gl + LPR * v;
+      if (q >= nvec) continue;
+      const size_t at = (size_t)u * a.ld + 4 * q;
+      float4 x = pu[v], o = unquad(apply_quad(a.eps, quad(pu[v]), quad(acc[v])));
+      if (MODE == MODE_RESID) {
+        const float4 y = ld_f4(a.Y + at);
+        const int cb = 4 * q;
+        o = make_float4(cb + 0 < a.kc ? y.x - o.x : 0.f, cb + 1 < a.kc ? y.y - o.y : 0.f,
+                        cb + 2 < a.kc ? y.z - o.z : 0.f, cb + 3 < a.kc ? y.w - o.w : 0.f);
+        x = o;
+      } else {
+        *reinterpret_cast<float4*>(a.AP + at) = o;
+      }
+      dot[v][0] = df_fma(dot[v][0], x.x, o.x);
+      dot[v][1] = df_fma(dot[v][1], x.y, o.y);
+      dot[v][2] = df_fma(dot[v][2], x.z, o.z);
+      dot[v][3] = df_fma(dot[v][3], x.w, o.w);
+    }
+  };
+  float4 pu[WIDE], acc[WIDE];
+  const int64_t nheavy = a.nheavy ? *a.nheavy : 0;
+  for (int64_t h = blockIdx.x; h < nheavy; h += gridDim.x) {
+    const int64_t u = a.heavy[h];
+    uint32_t j;
+    int len;
+    heavy_slice(a.row_ptr, u, gi, GPB, j, len);
+    load(u, pu, acc);
+    gather_wide<LPR, WIDE, WEIGHTED, false>(a, a.P, gl, ~0u, nvec, ~0u, j, len, pu, acc);
+#pragma unroll
+    for (int v = 0; v < WIDE; ++v) part[v][threadIdx.x] = acc[v];
+    __syncthreads();
+    if (gi == 0) {
+#pragma unroll
+      for (int v = 0; v < WIDE; ++v)
+        for (int g = 1; g < GPB; ++g) {
+          const float4 x = part[v][g * LPR + gl];
+          acc[v].x += x.x;
+          acc[v].y += x.y;
+          acc[v].z += x.z;
+          acc[v].w += x.w;
+        }
+      finish(u, pu, acc);
+    }
+    __syncthreads();
   }
+  for (int64_t u = (int64_t)blockIdx.x * GPB + gi; u < a.n; u += (int64_t)gridDim.x * GPB) {
+    uint32_t j, len;
+    row_slots(a.row_ptr, u, j, len);
+    if (len > (uint32_t)a.H) continue;
+    load(u, pu, acc);
+    gather_wide<LPR, WIDE, WEIGHTED, false>(a, a.P, gl, ~0u, nvec, ~0u, j, (int)len, pu, acc);
+    finish(u, pu, acc);
+  }
+  if (MODE == MODE_APPLY && a.pap_out == nullptr) return;
+  __syncthreads();
+  block_partials_groups<LPR, WIDE, WARPS, 256>(dot, sbuf, reinterpret_cast<float2*>(&part[0][0]),
+                                               a.ld);
+  finish_columns<MODE>(a, sbuf);
 }
 
 // ---------------------------------------------------------------------------- vector kernels
@@ -1040,8 +1143,10 @@ auto with_lpr(int nvec, F&& f) {
 }
 
 template <int MODE>
-const void* spmm_kernel(int nvec, bool weighted) {
-  return with_lpr(nvec, [&](auto lpr) -> const void* {
+const void* spmm_kernel(int64_t n, int ld, bool weighted) {
+  if (spmm_wide(n, ld))
+    return weighted ? (const void*)k_spmm_wide<true, MODE> : (const void*)k_spmm_wide<false, MODE>;
+  return with_lpr(ld / 4, [&](auto lpr) -> const void* {
     constexpr int LPR = decltype(lpr)::value;
     return weighted ? (const void*)k_spmm<LPR, true, MODE> : (const void*)k_spmm<LPR, false, MODE>;
   });
@@ -1058,7 +1163,7 @@ void spmm_shape(const erc_graph* g, int ld, int* grid, int32_t* H) {
   const int nvec = ld / 4;
   const int gpb = T / with_lpr(nvec, [](auto lpr) { return (int)decltype(lpr)::value; });
   const long long blocks = ((long long)g->n + gpb - 1) / gpb;
-  *grid = one_wave_grid(spmm_kernel<MODE_STEP>(nvec, g->val != nullptr), T, blocks);
+  *grid = one_wave_grid(spmm_kernel<MODE_STEP>(g->n, ld, g->val != nullptr), T, blocks);
   const long long groups = std::min<long long>(blocks, 3LL * sm_count()) * gpb;
   long long h = 2 * g->m / (8 * groups);
   if (h < 32) h = 32;
@@ -1080,6 +1185,15 @@ erc_status build_heavy(const erc_graph* g, int32_t H, const HeavyRows& hv, cudaS
 
 template <int MODE>
 erc_status launch_spmm(const SpmmArgs& a, int grid, cudaStream_t s) {
+  if (spmm_wide(a.n, a.ld)) {
+    if (a.val)
+      k_spmm_wide<true, MODE><<<grid, T, 0, s>>>(a);
+    else
+      k_spmm_wide<false, MODE><<<grid, T, 0, s>>>(a);
+    count_launches(1);
+    ERC_CUDA(cudaGetLastError());
+    return ERC_OK;
+  }
   return with_lpr(a.ld / 4, [&](auto lpr) -> erc_status {
     constexpr int LPR = decltype(lpr)::value;
     if (a.val)

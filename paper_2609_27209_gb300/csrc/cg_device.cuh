@@ -329,6 +329,60 @@ __device__ __forceinline__ Quad apply_quad(float eps, Quad pu, Quad acc) {
   return Quad{fma2(e, pu.a, acc.a), fma2(e, pu.b, acc.b)};
 }
 
+// acc[v] += w (p_u - p_v) over the CSR slots [j, j + len) of row u, for the lane's VPL quads of
+// every neighbour at once: rows of more than 128 columns.  The ids pass by shuffles, and 8 / VPL
+// neighbours are in flight.  A walk for each quad passes over the row bounds and ids twice and
+// waits twice (10,000 nodes, 256 columns: 60,000 edges 976 us a solve, 881 with both quads at once,
+// 875 before the walk; 120,000 edges 1,130, 901 and 890).
+template <int LPR, int VPL, bool WEIGHTED, bool L2ONLY>
+__device__ __forceinline__ void gather_wide(const SpmmArgs& a, const float* __restrict__ src,
+                                            int gl, unsigned gm, int nvec, unsigned on,
+                                            uint32_t j, int len,
+                                            const float4 (&pu)[VPL], float4 (&acc)[VPL]) {
+  constexpr int U = 8 / VPL;
+  for (int jb = 0; jb < len; jb += LPR) {
+    int32_t cidx = 0;
+    float wv = 1.f;
+    if (jb + gl < len) {
+      cidx = __ldg(a.col + (size_t)(j + (uint32_t)(jb + gl)));
+      if (WEIGHTED) wv = __ldg(a.val + (size_t)(j + (uint32_t)(jb + gl)));
+    }
+    const int cnt = min(LPR, len - jb);
+    for (int t = 0; t < cnt; t += U) {
+      int cj[U];
+      float wj[U];
+      float4 pv[U][VPL];
+#pragma unroll
+      for (int k = 0; k < U; ++k) {
+        cj[k] = __shfl_sync(gm, cidx, (t + k) & (LPR - 1), LPR);
+        wj[k] = WEIGHTED ? __shfl_sync(gm, wv, (t + k) & (LPR - 1), LPR) : 1.f;
+        if (t + k >= cnt) wj[k] = 0.f;
+      }
+#pragma unroll
+      for (int k = 0; k < U; ++k)
+#pragma unroll
+        for (int v = 0; v < VPL; ++v) {
+          const int q = gl + LPR * v;
+          const bool take = q < nvec && t + k < cnt && ((on >> v) & 1u);
+          const float* at = src + (size_t)cj[k] * a.ld + 4 * q;
+          if constexpr (L2ONLY)
+            pv[k][v] = ldcg_f4_if(take, at, pu[v]);
+          else
+            pv[k][v] = take ? ld_f4(at) : pu[v];
+        }
+#pragma unroll
+      for (int k = 0; k < U; ++k)
+#pragma unroll
+        for (int v = 0; v < VPL; ++v) {
+          acc[v].x = fmaf(wj[k], pu[v].x - pv[k][v].x, acc[v].x);
+          acc[v].y = fmaf(wj[k], pu[v].y - pv[k][v].y, acc[v].y);
+          acc[v].z = fmaf(wj[k], pu[v].z - pv[k][v].z, acc[v].z);
+          acc[v].w = fmaf(wj[k], pu[v].w - pv[k][v].w, acc[v].w);
+        }
+    }
+  }
+}
+
 // the vectors and per-column state of one batched solve
 struct VecArgs {
   int32_t n, ld, kc;
@@ -432,56 +486,6 @@ __host__ __device__ constexpr size_t resident_shared_floats(int hrows, int vpl) 
   return 4 * (size_t)PT * (size_t)(hrows * vpl);
 }
 
-// acc[v] += w (p_u - p_v) over the CSR slots [j, j + len) of row u, for the lane's VPL quads of
-// every neighbour at once: rows of more than 128 columns.  The ids pass by shuffles, and 8 / VPL
-// neighbours are in flight.  A walk for each quad passes over the row bounds and ids twice and
-// waits twice (10,000 nodes, 256 columns: 60,000 edges 976 us a solve, 881 with both quads at once,
-// 875 before the walk; 120,000 edges 1,130, 901 and 890).
-template <int LPR, int VPL, bool WEIGHTED>
-__device__ __forceinline__ void gather_wide(const SpmmArgs& a, const float* __restrict__ src,
-                                            int gl, unsigned gm, int nvec, unsigned on,
-                                            uint32_t j, int len,
-                                            const float4 (&pu)[VPL], float4 (&acc)[VPL]) {
-  constexpr int U = 8 / VPL;
-  for (int jb = 0; jb < len; jb += LPR) {
-    int32_t cidx = 0;
-    float wv = 1.f;
-    if (jb + gl < len) {
-      cidx = __ldg(a.col + (size_t)(j + (uint32_t)(jb + gl)));
-      if (WEIGHTED) wv = __ldg(a.val + (size_t)(j + (uint32_t)(jb + gl)));
-    }
-    const int cnt = min(LPR, len - jb);
-    for (int t = 0; t < cnt; t += U) {
-      int cj[U];
-      float wj[U];
-      float4 pv[U][VPL];
-#pragma unroll
-      for (int k = 0; k < U; ++k) {
-        cj[k] = __shfl_sync(gm, cidx, (t + k) & (LPR - 1), LPR);
-        wj[k] = WEIGHTED ? __shfl_sync(gm, wv, (t + k) & (LPR - 1), LPR) : 1.f;
-        if (t + k >= cnt) wj[k] = 0.f;
-      }
-#pragma unroll
-      for (int k = 0; k < U; ++k)
-#pragma unroll
-        for (int v = 0; v < VPL; ++v) {
-          const int q = gl + LPR * v;
-          pv[k][v] = ldcg_f4_if(q < nvec && t + k < cnt && ((on >> v) & 1u),
-                                src + (size_t)cj[k] * a.ld + 4 * q, pu[v]);
-        }
-#pragma unroll
-      for (int k = 0; k < U; ++k)
-#pragma unroll
-        for (int v = 0; v < VPL; ++v) {
-          acc[v].x = fmaf(wj[k], pu[v].x - pv[k][v].x, acc[v].x);
-          acc[v].y = fmaf(wj[k], pu[v].y - pv[k][v].y, acc[v].y);
-          acc[v].z = fmaf(wj[k], pu[v].z - pv[k][v].z, acc[v].z);
-          acc[v].w = fmaf(wj[k], pu[v].w - pv[k][v].w, acc[v].w);
-        }
-    }
-  }
-}
-
 // o = L_eps s on the rows r0 + i rstep, i < nrows, of s = src (n x ld): o_u = eps s_u +
 // sum_v w_uv (s_u - s_v).  own(u, v) is float4 slot v of the lane of s_u.  The rows heavier than
 // a.H (the ascending list hv[0..nh) of their i) are split over all groups of the block, hrows of
@@ -520,7 +524,7 @@ __device__ __forceinline__ void block_apply(const SpmmArgs& a, const float* src,
         int len;
         heavy_slice(a.row_ptr, u, gi, GPB, j, len);
         load(u, pu, acc);
-        gather_wide<LPR, VPL, WEIGHTED>(a, src, gl, gm, nvec, on, j, len, pu, acc);
+        gather_wide<LPR, VPL, WEIGHTED, true>(a, src, gl, gm, nvec, on, j, len, pu, acc);
 #pragma unroll
         for (int v = 0; v < VPL; ++v) part[(k * VPL + v) * PT + threadIdx.x] = acc[v];
       }
@@ -548,7 +552,7 @@ __device__ __forceinline__ void block_apply(const SpmmArgs& a, const float* src,
       row_slots(a.row_ptr, u, j, len);
       if (len > (uint32_t)a.H) continue;
       load(u, pu, acc);
-      gather_wide<LPR, VPL, WEIGHTED>(a, src, gl, gm, nvec, on, j, (int)len, pu, acc);
+      gather_wide<LPR, VPL, WEIGHTED, true>(a, src, gl, gm, nvec, on, j, (int)len, pu, acc);
       give(i, u, pu, acc);
     }
     return;
