@@ -201,9 +201,10 @@ __global__ void __launch_bounds__(T, 2) k_spmm(const __grid_constant__ SpmmArgs 
 // The operator for rows of 385 to 512 columns of a small block: a warp takes a row's four quads a
 // lane at once, two neighbours in flight.  Four slices of k_spmm each fill their pipeline anew, and
 // such graphs have only a few rows a group to spread that over.  512 columns: 20,000 nodes, 80,000
-// edges 41 us against 49 in slices; 3,000 nodes, 30,000 edges 26 against 31.  From P = 82 MB on the
-// slices are as fast or faster (40,000 nodes, 400,000 edges 136 against 131; 80,000 nodes,
-// 800,000 edges 360 against 253), as are three slices (384 columns, 20,000 nodes: 61 against 57).
+// edges 41 us against 49 in slices; 3,000 nodes, 30,000 edges 26 against 31.  At 82 MB it
+// depends on the degree (40,000 nodes: 160,000 edges 79 against 88, 400,000 edges 136 against 131),
+// and beyond the slices win (80,000 nodes, 800,000 edges 360 against 253), as three slices do from
+// 10,000 nodes on (384 columns, 20,000 nodes: 61 against 57).
 constexpr int WIDE = 4;  // quads a lane
 inline bool spmm_wide(int64_t n, int ld) {
   return ld > 384 && ld <= 512 && n * ld * 4 <= (int64_t(64) << 20);
